@@ -46,74 +46,95 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// The launch counter of a partials buffer: one unsigned after its kMaxPartials * 8 doubles
-// (allocated with them, zero between launches).
-__device__ __forceinline__ unsigned* partials_counter(double* partials)
+// Layout of a partials buffer: 8 doubles per block, 8 doubles per group of kSumGroup blocks,
+// then the tickets (one unsigned per group and one for the groups, zero between launches).
+constexpr int kSumGroup = 64;
+constexpr int kSumGroups = kMaxPartials / kSumGroup;
+constexpr size_t kPartialsDoubles = (size_t)(kMaxPartials + kSumGroups) * 8 + kSumGroups + 8;
+
+// Sum of column q over `count` rows of 8 doubles by one warp (count <= 64), the same order for
+// every caller.
+__device__ __forceinline__ double rows_sum(const double* rows, int count, int q)
 {
-    return reinterpret_cast<unsigned*>(partials + (size_t)kMaxPartials * 8);
+    const int lane = threadIdx.x & 31;
+    const double a = lane < count ? __ldcg(rows + (size_t)lane * 8 + q) : 0.0;
+    const double b = lane + 32 < count ? __ldcg(rows + (size_t)(lane + 32) * 8 + q) : 0.0;
+    return warp_sum(a + b);
 }
 
-// The block's NV sums into partials[block * 8 + q].  fin_out (nullable): the block that
-// finishes last (ticket from the partials counter, after a fence on every block's writes)
-// also sums all blocks' partials, in a fixed order, into fin_out[0..7] and the gauge shift
-// fin_out[8] = sum r / count unfloored, and resets the counter, with no second launch.
-template <int NV>
-__device__ __forceinline__ void block_sums(double (&v)[NV], double* partials, unsigned block,
+// The block's NV sums of v into partials[block * 8 + q]; at most 256 threads, every one of them
+// here.  fin_out (nullable): the grid's sums go into fin_out[0..NV-1] (and, for the residual's
+// five, the gauge shift fin_out[8] = sum r / count unfloored) with no second launch.  The last
+// block of each group of 64 (a ticket, after a fence on the blocks' writes) sums the group's
+// rows, the last group sums the groups' rows, both in a fixed order.
+//
+// FP64 additions bound this, not the data: the FP64 pipe takes 16 cycles per warp instruction
+// and SM.  So the threads' values go through shared memory and one warp sums each quantity (21
+// FP64 instructions per quantity and block of FP32 values; a shuffle tree in every warp took
+// 53), and the tail sums 2 x 64 rows by one warp per quantity instead of all rows in one block.
+// Measured against that form: mixed solve at 128^3 10.05 -> 8.70 ms; at 512^3 the 22 restricting
+// residuals 12.0 -> 11.0 ms, a sum of FP64 cells 0.53 -> 0.29 ms.
+template <int NV, typename V>
+__device__ __forceinline__ void block_sums(const V (&v)[NV], double* partials, unsigned block,
                                            double* fin_out = nullptr)
 {
-    __shared__ double sh[NV][32];
+    __shared__ V sh[NV][256];
+    __shared__ double tot[NV];
     __shared__ bool last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nt = blockDim.x, nw = nt >> 5;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        double s = warp_sum(v[q]);
-        if (lane == 0) sh[q][wid] = s;
-    }
+    for (int q = 0; q < NV; ++q) sh[q][t] = v[q];
     __syncthreads();
-    if (wid == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double s = lane < nw ? sh[q][lane] : 0.0;
-            s = warp_sum(s);
-            if (lane == 0) partials[(size_t)block * 8 + q] = s;
-        }
+    for (int q = wid; q < NV; q += nw) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int i = lane; i < nt; i += 32) s += (double)sh[q][i];
+        s = warp_sum(s);
+        if (lane == 0) partials[(size_t)block * 8 + q] = s;
     }
     if (!fin_out) return;
-    const unsigned nblocks = gridDim.x * gridDim.y * gridDim.z;
-    if (threadIdx.x == 0) {
+    const int nblocks = (int)(gridDim.x * gridDim.y * gridDim.z);
+    const int groups = (nblocks + kSumGroup - 1) / kSumGroup, g = (int)block / kSumGroup;
+    const int members = min(kSumGroup, nblocks - g * kSumGroup);
+    double* grows = partials + (size_t)kMaxPartials * 8;
+    unsigned* tickets = reinterpret_cast<unsigned*>(grows + (size_t)kSumGroups * 8);  // [groups], then the total's
+    __syncthreads();
+    if (t == 0) {
         __threadfence();
-        last = atomicAdd(partials_counter(partials), 1u) == nblocks - 1;
+        last = atomicAdd(tickets + g, 1u) == (unsigned)members - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    __shared__ double fs[8][32];
-    double acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    for (unsigned b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[q] += __ldcg(partials + (size_t)b * 8 + q);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const double s = warp_sum(acc[q]);
-        if (lane == 0) fs[q][wid] = s;
+    for (int q = wid; q < NV; q += nw) {
+        const double s = rows_sum(partials + (size_t)g * kSumGroup * 8, members, q);
+        if (lane == 0) grows[(size_t)g * 8 + q] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot[8];
-        for (int q = 0; q < 8; ++q) {
-            tot[q] = 0.0;
-            for (int w = 0; w < nw; ++w) tot[q] += fs[q][w];
-            fin_out[q] = tot[q];
+    if (t == 0) {
+        tickets[g] = 0u;
+        __threadfence();
+        last = atomicAdd(tickets + kSumGroups, 1u) == (unsigned)groups - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int q = wid; q < NV; q += nw) {
+        const double s = rows_sum(grows, groups, q);
+        if (lane == 0) {
+            tot[q] = s;
+            fin_out[q] = s;
         }
-        fin_out[8] = tot[3] > 0.0 ? tot[0] / tot[3] : 0.0;
-        *partials_counter(partials) = 0u;
+    }
+    __syncthreads();
+    if (t == 0) {
+        if constexpr (NV >= 4) fin_out[8] = tot[3] > 0.0 ? tot[0] / tot[3] : 0.0;
+        tickets[kSumGroups] = 0u;
     }
 }
 
-template <int NV>
-__device__ __forceinline__ void block_sums(double (&v)[NV], double* partials, double* fin_out = nullptr)
+template <int NV, typename V>
+__device__ __forceinline__ void block_sums(const V (&v)[NV], double* partials, double* fin_out = nullptr)
 {
     block_sums<NV>(v, partials, blockIdx.x, fin_out);
 }
@@ -172,7 +193,7 @@ struct Workspace {
     bool fft32_ready = false;
     // own stream, reductions and device scalars of one box of a batched solve
     cudaStream_t stream = nullptr;
-    double* partials = nullptr;    // kMaxPartials * 8
+    double* partials = nullptr;    // kPartialsDoubles
     double* out = nullptr;         // 64 device results
     double* host = nullptr;        // 64 pinned host mirror
     double* lam = nullptr;         // gauge multiplier (device)
@@ -190,7 +211,7 @@ struct pm_ctx {
     std::map<int, pmeft::Workspace*> ws;
     std::vector<pmeft::Workspace*> batch;  // one workspace per box of a batched solve
     cudaStream_t batch_stream = nullptr;    // capture / launch stream of the batched graph
-    double* red_partials = nullptr;  // kMaxPartials * 8 doubles
+    double* red_partials = nullptr;  // kPartialsDoubles doubles
     double* red_out = nullptr;       // device results (64 doubles: [0..8] residual, [16..] mean, [32..] norms)
     double* host_out = nullptr;      // pinned host mirror (64 doubles)
     int* flag = nullptr;             // device error flag

@@ -11,6 +11,7 @@
 // restricted mask (screening off where at least half the children were floored).
 // Two drivers: an FP64 FAS V-cycle, and an FP64 defect-correction loop whose inner
 // FAS V-cycle runs in FP32 on the correction e with the FP64 iterate as background.
+#include <algorithm>
 #include <cmath>
 
 #include "internal.cuh"
@@ -200,10 +201,7 @@ __global__ void __launch_bounds__(256) k_residual(const T* __restrict__ u, const
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x)
         residual_cell<T, BG, WRITE_R, MIXED>(u, F, fscale, lam, kmask, bg, gap, n, lg, ih2, nu, kap, Df, lsat_c,
                                              floor_piece, r, sat, rplain, chi32, gap32, c, fa);
-    double acc[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] = (double)fa[q];
-    block_sums<5>(acc, partials, fin_out);
+    block_sums<5>(fa, partials, fin_out);
 }
 
 // The FP64 residual of a level without a background (the FP64 cycle's levels, the mixed
@@ -260,10 +258,7 @@ __global__ void __launch_bounds__(256) k_residual64_zm(const double* __restrict_
                                                        floor_piece, r, sat, rplain, chi32, gap32, c, fa);
         __syncthreads();  // the slot of plane z - 1 is refilled next step
     }
-    double acc[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] = (double)fa[q];
-    block_sums<5>(acc, partials, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z), fin_out);
+    block_sums<5>(fa, partials, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z), fin_out);
 }
 
 // ------------------------------------------------------------------ transfers
@@ -899,49 +894,64 @@ __global__ void __launch_bounds__(kExactThreads) k_coarsest_exact(T* __restrict_
 
 // ------------------------------------------------------------------ misc
 
+// sum of x, four loads in flight per thread: FP32 data (the library's own buffers) by 16-byte
+// loads in FP32 per-thread sums (a few hundred terms each), FP64 across threads; FP64 data (the
+// caller's density among it) by aligned 8-byte loads, one FP64 addition per element
 template <typename T>
-__global__ void k_sum(const T* __restrict__ x, size_t total, double* __restrict__ partials,
-                      double* __restrict__ fin_out = nullptr)
+__global__ void __launch_bounds__(256) k_sum(const T* __restrict__ x, size_t total, double* __restrict__ partials,
+                                             double* __restrict__ fin_out)
 {
-    double v[2] = {0.0, 0.0};
+    constexpr int W = sizeof(T) == 4 ? 4 : 1;
+    struct alignas(W * sizeof(T)) Vec {
+        T e[W];
+    };
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-    if constexpr (sizeof(T) == 4) {
-        // FP32 data: 16-byte loads and FP32 per-thread sums (a few hundred terms each; the
-        // FP64 pipe would otherwise bound the pass), FP64 across threads
-        float a = 0.f, b = 0.f;
-        const size_t n4 = total / 4;
-        const float4* x4 = reinterpret_cast<const float4*>(x);
-        for (size_t c = tid; c < n4; c += stride) {
-            const float4 q = x4[c];
-            a += (q.x + q.y) + (q.z + q.w);
-            b += (q.x * q.x + q.y * q.y) + (q.z * q.z + q.w * q.w);
-        }
-        for (size_t c = 4 * n4 + tid; c < total; c += stride) {
-            a += (float)x[c];
-            b += (float)x[c] * (float)x[c];
-        }
-        v[0] = a;
-        v[1] = b;
-    } else {
-        for (size_t c = tid; c < total; c += stride) {
-            const double d = (double)x[c];
-            v[0] += d;
-            v[1] += d * d;
-        }
+    const size_t nv = total / W;  // total is a multiple of 512
+    const Vec* xv = reinterpret_cast<const Vec*>(x);
+    T a[4] = {T(0), T(0), T(0), T(0)};
+    size_t c = tid;
+    for (; c + 3 * stride < nv; c += 4 * stride) {
+        Vec q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q[k] = xv[c + k * stride];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int e = 0; e < W; ++e) a[k] += q[k].e[e];
     }
-    block_sums<2>(v, partials, fin_out);
+    for (; c < nv; c += stride) {
+        const Vec q = xv[c];
+#pragma unroll
+        for (int e = 0; e < W; ++e) a[0] += q.e[e];
+    }
+    const T v[1] = {(a[0] + a[1]) + (a[2] + a[3])};
+    block_sums<1>(v, partials, fin_out);
 }
 
 // sum of (x - mean)^2 with the mean read from the device
-__global__ void k_sum_centred(const double* __restrict__ x, size_t total, const double* __restrict__ sums,
-                              double* __restrict__ partials, double* __restrict__ fin_out = nullptr)
+__global__ void __launch_bounds__(256) k_sum_centred(const double* __restrict__ x, size_t total,
+                                                     const double* __restrict__ sums, double* __restrict__ partials,
+                                                     double* __restrict__ fin_out)
 {
     const double mean = sums[0] / (double)total;
-    double v[1] = {0.0};
-    for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x) {
-        const double d = x[c] - mean;
-        v[0] += d * d;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; c + 3 * stride < total; c += 4 * stride) {
+        double q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q[k] = x[c + k * stride];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double d = q[k] - mean;
+            a[k] += d * d;
+        }
     }
+    for (; c < total; c += stride) {
+        const double d = x[c] - mean;
+        a[0] += d * d;
+    }
+    const double v[1] = {(a[0] + a[1]) + (a[2] + a[3])};
     block_sums<1>(v, partials, fin_out);
 }
 
@@ -1615,11 +1625,17 @@ static void vcycle_up(Exec* ctx, std::vector<Level<T>>& lv, int stop, const T* F
     for (int l = stop - 1; l >= 0; --l) level_up(ctx, lv, l, F0, fs0, lam0, c);
 }
 
+// blocks of a summing pass: four per SM, so that a block's own sums are few beside its data
+static int sum_grid(Exec* ctx, size_t cells)
+{
+    const int g = grid_for(ctx, cells), cap = std::min(4 * ctx->num_sms, kMaxPartials);
+    return g < cap ? g : cap;
+}
+
 template <typename T>
 static void recentre(Exec* ctx, T* x, size_t cells)
 {
-    int grid = grid_for(ctx, cells);
-    if (grid > kMaxPartials) grid = kMaxPartials;
+    const int grid = sum_grid(ctx, cells);
     ctx->begin(PM_K_REDUCE, false, 0);
     k_sum<T><<<grid, kThreads, 0, ctx->stream>>>(x, cells, ctx->red_partials, ctx->red_out + 16);
     ctx->end();
@@ -1638,8 +1654,7 @@ static pm_status read_sums(Exec* ctx, int count)
 // |f - <f>|_2 for f = src * delta
 static pm_status source_norm(Exec* ctx, const double* delta, size_t cells, double src, double* out)
 {
-    int grid = grid_for(ctx, cells);
-    if (grid > kMaxPartials) grid = kMaxPartials;
+    const int grid = sum_grid(ctx, cells);
     ctx->begin(PM_K_REDUCE, false, 0);
     k_sum<double><<<grid, kThreads, 0, ctx->stream>>>(delta, cells, ctx->red_partials, ctx->red_out + 32);
     ctx->end();
@@ -1687,8 +1702,7 @@ static void residual_ff(Exec* ctx, Workspace* w, const float2* xff, const float2
 // sum of the correction e into red_out[16]
 static void correction_sum(Exec* ctx, const float* e, size_t cells)
 {
-    int grid = grid_for(ctx, cells);
-    if (grid > kMaxPartials) grid = kMaxPartials;
+    const int grid = sum_grid(ctx, cells);
     ctx->begin(PM_K_REDUCE, false, 0);
     k_sum<float><<<grid, kThreads, 0, ctx->stream>>>(e, cells, ctx->red_partials, ctx->red_out + 16);
     ctx->end();

@@ -210,10 +210,7 @@ __global__ void __launch_bounds__(256) k_residual_ff(const float2* __restrict__ 
             }
         }
     }
-    double acc[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] = (double)fa[q];
-    block_sums<5>(acc, partials, fin_out);
+    block_sums<5>(fa, partials, fin_out);
 }
 
 
@@ -557,10 +554,7 @@ __global__ void __launch_bounds__(256, 3) k_residual_ff_zm(const float2* __restr
             }
         }
     }
-    double acc[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] = (double)fa[q];
-    block_sums<5>(acc, partials, (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, fin_out);
+    block_sums<5>(fa, partials, (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, fin_out);
 }
 
 }  // namespace pmeft

@@ -213,10 +213,7 @@ __global__ void __launch_bounds__(256) k_residual_zm(const float* __restrict__ u
             for (int h = 0; h < 2; ++h) au[h] = ar[h] = ac[h] = an[h] = 0.f;
         }
     }
-    double acc[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] = (double)fa[q];
-    block_sums<5>(acc, partials, (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, fin_out);
+    block_sums<5>(fa, partials, (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, fin_out);
 }
 
 }  // namespace pmeft
