@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_batch_coarse(CoopParams P)
             const CoopBox& B = P.boxes[b];
             const CoopLevel& L = B.lv[l];
             coarsest_block<float, true>(L.u[0], L.f, 1.f, L.kmask, L.bg, L.n, (double)L.n * (double)L.n, B.nu_d,
-                                        B.kap_d, P.eta, P.coarse_sweeps, false, csm);
+                                        B.kap_d, P.eta, P.coarse_sweeps, false, csm, K64{});
             __syncthreads();
         }
         cur[l] = 0;

@@ -15,6 +15,7 @@
 #include <cmath>
 
 #include "internal.cuh"
+#include "cell64.cuh"
 #include "sweep_fused.cuh"
 #include "sweep_pair.cuh"
 #include "sweep_col.cuh"
@@ -204,63 +205,6 @@ __global__ void __launch_bounds__(256) k_residual(const T* __restrict__ u, const
     block_sums<5>(fa, partials, fin_out);
 }
 
-// The FP64 residual of a level without a background (the FP64 cycle's levels, the mixed
-// loops' confirming residual and the FP64 outer loop), marching up z: a block of 32 x 8
-// threads keeps three planes of its 32 x 8 tile and their one-cell halo in a shared ring, so
-// each iterate value is read from global memory once per block instead of once per stencil
-// point.  Arithmetic and sums as k_residual (residual_cell_s); grid (n/32, n/8, n/nz).
-constexpr int kR64TX = 32, kR64TY = 8;
-template <bool WRITE_R, bool MIXED>
-__global__ void __launch_bounds__(256) k_residual64_zm(const double* __restrict__ u, const double* __restrict__ F,
-                                                       double fscale, double lam, const uint8_t* __restrict__ kmask,
-                                                       int n, int nz, double ih2, double nu, double kap, double Df,
-                                                       double lsat_c, bool floor_piece, double* __restrict__ r,
-                                                       uint8_t* __restrict__ sat, double* __restrict__ partials,
-                                                       float* __restrict__ rplain, float* __restrict__ chi32,
-                                                       float* __restrict__ gap32, const double* __restrict__ lamp,
-                                                       double* __restrict__ fin_out)
-{
-    constexpr int WX = kR64TX + 2, WY = kR64TY + 2, PL = WX * WY;
-    __shared__ double ring[3][PL];
-    if (lamp) lam += *lamp;
-    const int m = n - 1;
-    const int x0 = blockIdx.x * kR64TX, y0 = blockIdx.y * kR64TY, z0 = blockIdx.z * nz;
-    const int t = threadIdx.x, tx = t & (kR64TX - 1), ty = t / kR64TX;
-    const size_t plane = (size_t)n * n;
-    auto load = [&](int z, int slot) {
-        const size_t zo = (size_t)(z & m) * plane;
-        for (int e = t; e < PL; e += 256) {
-            const int xx = e % WX, yy = e / WX;
-            ring[slot][e] = u[zo + (size_t)((y0 - 1 + yy) & m) * n + ((x0 - 1 + xx) & m)];
-        }
-    };
-    float fa[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    load(z0 - 1, 0);
-    load(z0, 1);
-    const int cl = (ty + 1) * WX + tx + 1;
-    for (int s = 0; s < nz; ++s) {
-        const int z = z0 + s;
-        load(z + 1, (s + 2) % 3);
-        __syncthreads();
-        const double* pm = ring[s % 3];        // plane z - 1
-        const double* pc = ring[(s + 1) % 3];  // plane z
-        const double* pp = ring[(s + 2) % 3];  // plane z + 1
-        Stencil<double> st, b;
-        st.c0 = pc[cl];
-        st.ax = pc[cl + 1] + pc[cl - 1];
-        st.ay = pc[cl + WX] + pc[cl - WX];
-        st.az = pp[cl] + pm[cl];
-        st.exy = pc[cl + 1 + WX] - pc[cl + 1 - WX] - pc[cl - 1 + WX] + pc[cl - 1 - WX];
-        st.exz = pp[cl + 1] - pm[cl + 1] - pp[cl - 1] + pm[cl - 1];
-        st.eyz = pp[cl + WX] - pm[cl + WX] - pp[cl - WX] + pm[cl - WX];
-        const size_t c = (size_t)z * plane + (size_t)(y0 + ty) * n + (x0 + tx);
-        residual_cell_s<double, false, WRITE_R, MIXED>(st, b, F, fscale, lam, kmask, nullptr, ih2, nu, kap, Df, lsat_c,
-                                                       floor_piece, r, sat, rplain, chi32, gap32, c, fa);
-        __syncthreads();  // the slot of plane z - 1 is refilled next step
-    }
-    block_sums<5>(fa, partials, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z), fin_out);
-}
-
 // ------------------------------------------------------------------ transfers
 
 // Coarse cell c = average of its 8 children, for the iterate (-> ur and the coarse start
@@ -342,7 +286,7 @@ __device__ __forceinline__ void fas_rhs_cell(const T* uc, const T* rc,
                                              uint8_t* kmask, const T* bg, int n, int lg,
                                              T ih2, T nu, T kap, T* fc, uint32_t* coefo,
                                              float* gapo, float lsat, bool apply_gm, T gm, size_t total,
-                                             size_t c)
+                                             size_t c, const K64* k64 = nullptr, const KW64* tab = nullptr)
 {
     const int i = (int)(c & (size_t)(n - 1));  // n is a power of two
     const size_t row = c >> lg;
@@ -355,6 +299,10 @@ __device__ __forceinline__ void fas_rhs_cell(const T* uc, const T* rc,
         const uint8_t kb = kmask[c];
         rcv -= gm * (T)(kb >> 4) * T(0.125);
         kmask[c] = kb & 15;
+    }
+    if constexpr (sizeof(T) == 8) {  // N + r with the FP64 cell's arithmetic (no background there)
+        fc[c] = eval64(s, k64->nu1, k64->ep0, tab[min((int)kmask[c], 8)], -rcv).G;
+        return;
     }
     const T w = screen_w<T>(kmask, c);
     const T kc = kap * w;
@@ -374,14 +322,20 @@ template <typename T, bool BG>
 __global__ void __launch_bounds__(256) k_fas_rhs(const T* __restrict__ uc, const T* __restrict__ rc,
                                                  uint8_t* __restrict__ kmask, const T* __restrict__ bg, int n,
                                                  T ih2, T nu, T kap, T* __restrict__ fc, uint32_t* __restrict__ coefo,
-                                                 float* __restrict__ gapo, float lsat, const double* __restrict__ gm_ptr)
+                                                 float* __restrict__ gapo, float lsat, const double* __restrict__ gm_ptr,
+                                                 K64 k64 = {})
 {
+    __shared__ KW64 tab[sizeof(T) == 8 ? 9 : 1];
+    if constexpr (sizeof(T) == 8) {
+        fill_kw64(tab, k64);
+        __syncthreads();
+    }
     const T gm = gm_ptr ? (T)(*gm_ptr) : T(0);
     const size_t total = (size_t)n * n * n;
     const int lg = __ffs(n) - 1;
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x)
         fas_rhs_cell<T, BG>(uc, rc, kmask, bg, n, lg, ih2, nu, kap, fc, coefo, gapo, lsat, gm_ptr != nullptr, gm, total,
-                            c);
+                            c, &k64, tab);
 }
 
 // k_fas_rhs for levels of at least 32^3, tiled: a block stages the iterate (and the
@@ -393,11 +347,13 @@ __global__ void __launch_bounds__(256) k_fas_rhs_tile(const T* __restrict__ uc, 
                                                       uint8_t* __restrict__ kmask, const T* __restrict__ bg, int n,
                                                       T ih2, T nu, T kap, T* __restrict__ fc,
                                                       uint32_t* __restrict__ coefo, float* __restrict__ gapo,
-                                                      float lsat, const double* __restrict__ gm_ptr)
+                                                      float lsat, const double* __restrict__ gm_ptr, K64 k64 = {})
 {
     constexpr int BX = 32, BY = 4, BZ = 4, WX = BX + 2, WY = BY + 2, WZ = BZ + 2, WXY = WX * WY, P = WXY * WZ;
     __shared__ T su[P];
     __shared__ T sb[BG ? P : 1];
+    __shared__ KW64 tab[sizeof(T) == 8 ? 9 : 1];
+    if constexpr (sizeof(T) == 8) fill_kw64(tab, k64);
     const int m = n - 1;
     const int X0 = blockIdx.x * BX, Y0 = blockIdx.y * BY, Z0 = blockIdx.z * BZ;
     for (int e = threadIdx.x; e < P; e += 256) {
@@ -435,6 +391,10 @@ __global__ void __launch_bounds__(256) k_fas_rhs_tile(const T* __restrict__ uc, 
             rcv -= gm * (T)(kb >> 4) * T(0.125);
             kmask[c] = kb & 15;
         }
+        if constexpr (sizeof(T) == 8) {
+            fc[c] = eval64(s, k64.nu1, k64.ep0, tab[min((int)kmask[c], 8)], -rcv).G;
+            continue;
+        }
         const T w = screen_w<T>(kmask, c);
         const T kc = kap * w;
         Local<T> o = local_eval<T, BG>(s, b, ih2, nu, kc, T(0), T(0));
@@ -450,6 +410,47 @@ __global__ void __launch_bounds__(256) k_fas_rhs_tile(const T* __restrict__ uc, 
     }
 }
 
+// The eight children of a coarse cell from its 3x3x3 neighbourhood d, interpolated separably
+// (weights 3/4 and 1/4 per axis) and handed out as x pairs: put(dz, dy, o0, o1, scale).  FP64
+// values, whose pipe is the limit, come as 64 times the children (3 v1 + v0 per axis is one fused
+// multiply-add; the power of two is exact) with scale 1/64: 46 FP64 instructions for eight
+// children where the weighted form takes 84.
+template <typename T, typename Put>
+__device__ __forceinline__ void prolong_children(const T (&d)[3][3][3], Put&& put)
+{
+    auto mix = [](T near, T far) {
+        if constexpr (sizeof(T) == 8) return fma(3.0, near, far);
+        else return T(0.75) * near + T(0.25) * far;
+    };
+    T px[3][3][2], py[3][2][2];
+#pragma unroll
+    for (int kz = 0; kz < 3; ++kz) {
+#pragma unroll
+        for (int jy = 0; jy < 3; ++jy) {
+            px[kz][jy][0] = mix(d[kz][jy][1], d[kz][jy][0]);
+            px[kz][jy][1] = mix(d[kz][jy][1], d[kz][jy][2]);
+        }
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+            for (int dx = 0; dx < 2; ++dx) py[kz][dy][dx] = mix(px[kz][1][dx], px[kz][dy ? 2 : 0][dx]);
+    }
+#pragma unroll
+    for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy)
+            put(dz, dy, mix(py[1][dy][0], py[dz ? 2 : 0][dy][0]), mix(py[1][dy][1], py[dz ? 2 : 0][dy][1]),
+                sizeof(T) == 8 ? T(1.0 / 64.0) : T(1));
+}
+
+// fine value plus a child's correction
+template <typename T>
+__device__ __forceinline__ T prolong_apply(T o, T scale, T fine)
+{
+    if constexpr (sizeof(T) == 8) return fma(o, scale, fine);
+    else return fine + o;
+}
+
 // fine += trilinear cell-centred prolongation of (uc - ur), periodic.  One thread per
 // coarse cell writes its 8 children: the 3x3x3 coarse neighbourhood is interpolated
 // separably (weights 3/4 and 1/4 per axis, i.e. 27/64, 9/64, 3/64, 1/64 in 3D), and the
@@ -459,43 +460,27 @@ __device__ __forceinline__ void prolong_add_cell(const T* uc, const T* ur, int n
                                                  T* uf, size_t c)
 {
     const int nf = 2 * nc, mc = nc - 1;
-    const T a = T(0.75), b = T(0.25);
     const int I = (int)(c & (size_t)mc);  // nc is a power of two
     const size_t row = c >> lgc;
     const int J = (int)(row & (size_t)mc), K = (int)(row >> lgc);
     const int xs[3] = {(I - 1) & mc, I, (I + 1) & mc};
     const int ys[3] = {(J - 1) & mc, J, (J + 1) & mc};
     const int zs[3] = {(K - 1) & mc, K, (K + 1) & mc};
-    // along x: px[z][y][child]
-    T px[3][3][2];
+    T d[3][3][3];
 #pragma unroll
     for (int kz = 0; kz < 3; ++kz)
 #pragma unroll
         for (int jy = 0; jy < 3; ++jy) {
             const size_t base = ((size_t)zs[kz] * nc + ys[jy]) * nc;
-            T v[3];
 #pragma unroll
-            for (int ix = 0; ix < 3; ++ix) v[ix] = ur ? uc[base + xs[ix]] - ur[base + xs[ix]] : uc[base + xs[ix]];
-            px[kz][jy][0] = a * v[1] + b * v[0];
-            px[kz][jy][1] = a * v[1] + b * v[2];
+            for (int ix = 0; ix < 3; ++ix)
+                d[kz][jy][ix] = ur ? uc[base + xs[ix]] - ur[base + xs[ix]] : uc[base + xs[ix]];
         }
-    // along y, then z, then add to the children
-#pragma unroll
-    for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy) {
-            T out[2];
-#pragma unroll
-            for (int dx = 0; dx < 2; ++dx) {
-                T py[3];
-#pragma unroll
-                for (int kz = 0; kz < 3; ++kz) py[kz] = a * px[kz][1][dx] + b * px[kz][dy ? 2 : 0][dx];
-                out[dx] = a * py[1] + b * py[dz ? 2 : 0];
-            }
-            T* f = uf + ((size_t)(2 * K + dz) * nf + (2 * J + dy)) * nf + 2 * I;
-            f[0] += out[0];
-            f[1] += out[1];
-        }
+    prolong_children<T>(d, [&](int dz, int dy, T o0, T o1, T s) {
+        T* f = uf + ((size_t)(2 * K + dz) * nf + (2 * J + dy)) * nf + 2 * I;
+        f[0] = prolong_apply<T>(o0, s, f[0]);
+        f[1] = prolong_apply<T>(o1, s, f[1]);
+    });
 }
 
 template <typename T>
@@ -527,65 +512,56 @@ __global__ void __launch_bounds__(256) k_prolong_add_tile(const T* __restrict__ 
         sd[e] = ur ? uc[g] - ur[g] : uc[g];
     }
     __syncthreads();
-    const T a = T(0.75), b = T(0.25);
     const int x = threadIdx.x & 31, y = (threadIdx.x >> 5) & 3;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int z = (threadIdx.x >> 7) + 2 * h;
-        T px[3][3][2];
+        T d[3][3][3];
 #pragma unroll
         for (int kz = 0; kz < 3; ++kz)
 #pragma unroll
-            for (int jy = 0; jy < 3; ++jy) {
-                const T* v = sd + ((z + kz) * WY + (y + jy)) * WX + x;
-                px[kz][jy][0] = a * v[1] + b * v[0];
-                px[kz][jy][1] = a * v[1] + b * v[2];
-            }
+            for (int jy = 0; jy < 3; ++jy)
+#pragma unroll
+                for (int ix = 0; ix < 3; ++ix) d[kz][jy][ix] = sd[((z + kz) * WY + (y + jy)) * WX + x + ix];
         const int I = X0 + x, J = Y0 + y, K = Z0 + z;
-#pragma unroll
-        for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-            for (int dy = 0; dy < 2; ++dy) {
-                T out[2];
-#pragma unroll
-                for (int dx = 0; dx < 2; ++dx) {
-                    T py[3];
-#pragma unroll
-                    for (int kz = 0; kz < 3; ++kz) py[kz] = a * px[kz][1][dx] + b * px[kz][dy ? 2 : 0][dx];
-                    out[dx] = a * py[1] + b * py[dz ? 2 : 0];
-                }
-                T* f = uf + ((size_t)(2 * K + dz) * nf + (2 * J + dy)) * nf + 2 * I;
-                f[0] += out[0];
-                f[1] += out[1];
-            }
+        prolong_children<T>(d, [&](int dz, int dy, T o0, T o1, T s) {
+            T* f = uf + ((size_t)(2 * K + dz) * nf + (2 * J + dy)) * nf + 2 * I;
+            f[0] = prolong_apply<T>(o0, s, f[0]);
+            f[1] = prolong_apply<T>(o1, s, f[1]);
+        });
     }
 }
 
 // ------------------------------------------------------------------ coarsest level
 
-// Exact-enough solve of the coarsest level (at most 8^3 cells) in one thread block, in the
+// Exact-enough solve of the coarsest level (at most 8^3 cells) in one thread block of 256, in the
 // storage type's arithmetic (FP64 for the FP64 cycle, FP32 inside the FP32 inner cycle):
 // `sweeps` red-black sweeps, each followed by the gauge update lambda -= sum r / #unfloored.
-// The block sums go through warp shuffles and one exchange between the warps.
+// A latency chain, so it is kept short: a thread owns one red and one black cell (threads beyond
+// half the cells idle), whose neighbour offsets, background stencils, weights and right-hand sides
+// stay in registers for all sweeps; it holds its new value until every thread has read its
+// neighbours, so a half-sweep is one evaluation and two barriers with no copy of the field; and
+// levels of at most 64 cells (the default 4^3) are solved by one warp, whose barriers are free.
+// The 4^3 launch: FP64 88 -> 60 us (the latency of dependent FP64 operations), FP32 16.5 -> 10.4.
 template <typename T>
 struct CoarsestSmem {
-    T su[512], ss[512], sf[512], sb[512];
+    T su[512], sf[512], sb[512];
     uint8_t sk[512];
     T red[2][8];
+    KW64 tab[9];
 };
 
 // The coarsest solve of one level (at most 8^3 cells) by the calling block, its arrays in sm.
 template <typename T, bool BG>
 __device__ void coarsest_block(T* u, const T* F, T fscale, const uint8_t* kmask,
                                const T* bg, int n, double ih2_d, double nu_d, double kap_d, double eta,
-                               int sweeps, bool floor_piece, CoarsestSmem<T>& sm)
+                               int sweeps, bool floor_piece, CoarsestSmem<T>& sm, const K64& k64)
 {
     T* su = sm.su;
-    T* ss = sm.ss;
     T* sf = sm.sf;
     T* sb = sm.sb;
     uint8_t* sk = sm.sk;
-    const int cells = n * n * n, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int cells = n * n * n, t = threadIdx.x, lane = t & 31, wid = t >> 5, lg = __ffs(n) - 1;
     const T ih2 = (T)ih2_d, nu = (T)nu_d, kap = (T)kap_d;
     for (int c = t; c < cells; c += blockDim.x) {
         su[c] = u[c];
@@ -593,71 +569,123 @@ __device__ void coarsest_block(T* u, const T* F, T fscale, const uint8_t* kmask,
         sk[c] = kmask ? kmask[c] : 0;
         sb[c] = BG ? bg[c] : T(0);
     }
+    if constexpr (sizeof(T) == 8) fill_kw64(sm.tab, k64);
     __syncthreads();
     const T sp = nu >= T(0) ? T(-1) : T(1);
     const double sqDf = eta * 6.0 * fabs(nu_d) * ih2_d;
     const T Df = (T)(sqDf * sqDf);
     const T lsat_c = kap != T(0) ? (T)(0.75 * nu_d * (1.0 - eta) / kap_d) : T(0);  // L_sat
+    const bool one = cells <= 64;  // one warp works, the others wait at the end
+    const int nt = one ? 32 : (int)blockDim.x;
+    auto sync = [&]() {
+        if (one) __syncwarp();
+        else __syncthreads();
+    };
+    const bool mine = t < (cells >> 1);
+    // the thread's red (q = 0) and black (q = 1) cell
+    int c[2], o[2][6];
+    Stencil<T> b[2];
+    T kc[2], lsat[2], f[2];
+    KW64 w64[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int h = mine ? t : 0;
+        const int m = h & ((n >> 1) - 1), row = h >> (lg - 1), j = row & (n - 1), k = row >> lg;
+        const int i = 2 * m + ((j + k + q) & 1), nn = n * n;
+        c[q] = row * n + i;
+        o[q][0] = ((i + 1) & (n - 1)) - i;
+        o[q][1] = ((i - 1) & (n - 1)) - i;
+        o[q][2] = (((j + 1) & (n - 1)) - j) * n;
+        o[q][3] = (((j - 1) & (n - 1)) - j) * n;
+        o[q][4] = (((k + 1) & (n - 1)) - k) * nn;
+        o[q][5] = (((k - 1) & (n - 1)) - k) * nn;
+        if (BG) b[q] = load_stencil<T>(sb, sb, i, j, k, n);
+        const int kb = sk[c[q]];
+        f[q] = sf[c[q]];
+        if constexpr (sizeof(T) == 8) {
+            w64[q] = sm.tab[min(kb, 8)];
+        } else {
+            const T w = kb >= 8 ? T(0) : (T)(8 - kb) * T(0.125);
+            kc[q] = kap * w;
+            lsat[q] = kc[q] != T(0) ? (kmask ? lsat_c / w : lsat_c) : T(0);
+        }
+    }
+    auto stencil = [&](int q) {  // load_stencil's sums
+        const T* p = su + c[q];
+        const int xp = o[q][0], xm = o[q][1], yp = o[q][2], ym = o[q][3], zp = o[q][4], zm = o[q][5];
+        Stencil<T> s;
+        s.c0 = p[0];
+        s.ax = p[xp] + p[xm];
+        s.ay = p[yp] + p[ym];
+        s.az = p[zp] + p[zm];
+        s.exy = p[xp + yp] - p[xp + ym] - p[xm + yp] + p[xm + ym];
+        s.exz = p[xp + zp] - p[xp + zm] - p[xm + zp] + p[xm + zm];
+        s.eyz = p[yp + zp] - p[yp + zm] - p[ym + zp] + p[ym + zm];
+        return s;
+    };
     T lam = T(0);
-    for (int it = 0; it < sweeps; ++it) {
-        for (int colour = 0; colour < 2; ++colour) {
-            for (int c = t; c < cells; c += blockDim.x) ss[c] = su[c];
-            __syncthreads();
-            for (int c = t; c < cells; c += blockDim.x) {
-                const int i = c % n, j = (c / n) % n, k = c / (n * n);
-                if (((i + j + k) & 1) != colour) continue;
-                Stencil<T> s = load_stencil<T>(ss, ss, i, j, k, n);
-                Stencil<T> b;
-                if (BG) b = load_stencil<T>(sb, sb, i, j, k, n);
-                const T w = sk[c] >= 8 ? T(0) : (T)(8 - sk[c]) * T(0.125);
-                const T kc = kap * w;
-                Local<T> o = local_eval<T, BG>(s, b, ih2, nu, kc, sf[c] + lam, kc != T(0) ? (kmask ? lsat_c / w : lsat_c) : T(0));
-                su[c] = s.c0 + local_update(o, sp, Df, ih2);
-            }
-            __syncthreads();
+    for (int it = 0; it < sweeps && t < nt; ++it) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const Stencil<T> s = stencil(q);
+            T v;
+            if constexpr (sizeof(T) == 8)
+                v = s.c0 + update64(eval64(s, k64.nu1, k64.ep0, w64[q], f[q] + lam), k64, w64[q]);
+            else
+                v = s.c0 + local_update(local_eval<T, BG>(s, b[q], ih2, nu, kc[q], f[q] + lam, lsat[q]), sp, Df, ih2);
+            sync();
+            if (mine) su[c[q]] = v;
+            sync();
         }
         // gauge update from the residual
         T a0 = T(0), a1 = T(0);
-        for (int c = t; c < cells; c += blockDim.x) {
-            const int i = c % n, j = (c / n) % n, k = c / (n * n);
-            Stencil<T> s = load_stencil<T>(su, su, i, j, k, n);
-            Stencil<T> b;
-            if (BG) b = load_stencil<T>(sb, sb, i, j, k, n);
-            const T w = sk[c] >= 8 ? T(0) : (T)(8 - sk[c]) * T(0.125);
-            const T kc = kap * w;
-            Local<T> o = local_eval<T, BG>(s, b, ih2, nu, kc, sf[c] + lam, kc != T(0) ? (kmask ? lsat_c / w : lsat_c) : T(0));
-            const bool fl = (o.P != T(0)) && (o.D < (floor_piece ? Df : T(0)));
-            a0 += fl ? nu * o.g : -o.G;
-            a1 += fl ? T(0) : T(1);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const Stencil<T> s = stencil(q);
+            bool fl;
+            T rv;
+            if constexpr (sizeof(T) == 8) {
+                rv = resid64(eval64(s, k64.nu1, k64.ep0, w64[q], f[q] + lam), k64, w64[q],
+                             floor_piece ? k64.Df : 0.0, fl);
+            } else {
+                const Local<T> e = local_eval<T, BG>(s, b[q], ih2, nu, kc[q], f[q] + lam, lsat[q]);
+                fl = (e.P != T(0)) && (e.D < (floor_piece ? Df : T(0)));
+                rv = fl ? nu * e.g : -e.G;
+            }
+            a0 += mine ? rv : T(0);
+            a1 += mine && !fl ? T(1) : T(0);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            a0 += __shfl_down_sync(0xffffffffu, a0, o);
-            a1 += __shfl_down_sync(0xffffffffu, a1, o);
+        for (int d = 16; d > 0; d >>= 1) {
+            a0 += __shfl_xor_sync(0xffffffffu, a0, d);
+            a1 += __shfl_xor_sync(0xffffffffu, a1, d);
         }
-        if (lane == 0) {
-            sm.red[0][wid] = a0;
-            sm.red[1][wid] = a1;
+        if (!one) {
+            if (lane == 0) {
+                sm.red[0][wid] = a0;
+                sm.red[1][wid] = a1;
+            }
+            __syncthreads();
+            a0 = a1 = T(0);
+            for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {  // every thread, the same order
+                a0 += sm.red[0][q];
+                a1 += sm.red[1][q];
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        T s0 = T(0), s1 = T(0);
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {  // every thread, the same order
-            s0 += sm.red[0][q];
-            s1 += sm.red[1][q];
-        }
-        if (s1 > T(0)) lam -= s0 / s1;
-        __syncthreads();
+        if (a1 > T(0)) lam -= a0 / a1;
     }
-    for (int c = t; c < cells; c += blockDim.x) u[c] = su[c];
+    __syncthreads();
+    for (int q = t; q < cells; q += blockDim.x) u[q] = su[q];
 }
 
 template <typename T, bool BG>
 __global__ void __launch_bounds__(256) k_coarsest(T* __restrict__ u, const T* __restrict__ F, T fscale,
                                                   const uint8_t* __restrict__ kmask, const T* __restrict__ bg, int n,
                                                   double ih2_d, double nu_d, double kap_d, double eta, int sweeps,
-                                                  bool floor_piece)
+                                                  bool floor_piece, K64 k64)
 {
     __shared__ CoarsestSmem<T> sm;
-    coarsest_block<T, BG>(u, F, fscale, kmask, bg, n, ih2_d, nu_d, kap_d, eta, sweeps, floor_piece, sm);
+    coarsest_block<T, BG>(u, F, fscale, kmask, bg, n, ih2_d, nu_d, kap_d, eta, sweeps, floor_piece, sm, k64);
 }
 
 // ------------------------------------------------------------------ exact coarsest solve
@@ -1208,6 +1236,15 @@ static int tuned_cfg(Exec* ctx, Level<float>& L, const float* F, float fscale, f
     return best;
 }
 
+// Threads per block of an FP64 launch over `work` cells: 256, or fewer where that leaves less than
+// four blocks per SM, so that the cells spread over all SMs (k_half_sweep64 says why)
+static int thin_threads(Exec* x, size_t work)
+{
+    int t = kThreads;
+    while (t > 32 && work < (size_t)t * 4 * x->num_sms) t >>= 1;
+    return t;
+}
+
 // One red-black sweep as two half-sweep launches (one per colour), out of place: A = u[cur]
 // is read, B = u[1 - cur] receives the new values, then cur flips.
 template <typename T>
@@ -1233,17 +1270,26 @@ static void sweep_halves(Exec* ctx, Level<T>& L, const T* F, T fscale, T lam, co
             ctx->end();
         } else {
             ctx->begin(sizeof(T) == 8 ? PM_K_SWEEP64 : PM_K_SWEEP32, L.fine, (long long)(L.cells / 2));
-            // Method II where the parameters ask for it (the FP64 cycle; FP32 levels keep Method I)
-            const bool ops = sizeof(T) == 8 && ctx->prm.smoother == 1;
-            const T etanu = (T)(c.eta * std::fabs(c.nu));
-            if (ops)
-                k_half_sweep<T, false, true><<<grid, kThreads, 0, ctx->stream>>>(
-                    own, oth, B, F, fscale, lam, L.kmask, nullptr, nullptr, n, colour, h2inv, (T)c.nu, (T)c.kap, sp,
-                    (T)(sqDf * sqDf), lsn, L.lamp, etanu);
-            else
+            if constexpr (sizeof(T) == 8) {
+                // Method II where the parameters ask for it (the FP64 cycle; FP32 levels keep Method I)
+                const K64 k = make_k64(n, c.nu, c.kap, c.eta);
+                const size_t half = L.cells / 2;
+                const int th = thin_threads(ctx, half), gb = (int)((half + th - 1) / th);
+                if (ctx->prm.smoother == 1)
+                    k_half_sweep<T, false, true><<<grid, kThreads, 0, ctx->stream>>>(
+                        own, oth, B, F, fscale, lam, L.kmask, nullptr, nullptr, n, colour, h2inv, (T)c.nu, (T)c.kap,
+                        sp, (T)(sqDf * sqDf), lsn, L.lamp, (T)(c.eta * std::fabs(c.nu)));
+                else if (L.kmask)
+                    k_half_sweep64<true><<<gb, th, 0, ctx->stream>>>(own, oth, B, F, fscale, lam, L.kmask, n,
+                                                                     __builtin_ctz(n), colour, k, L.lamp);
+                else
+                    k_half_sweep64<false><<<gb, th, 0, ctx->stream>>>(own, oth, B, F, fscale, lam, nullptr, n,
+                                                                      __builtin_ctz(n), colour, k, L.lamp);
+            } else {
                 k_half_sweep<T, false><<<grid, kThreads, 0, ctx->stream>>>(
                     own, oth, B, F, fscale, lam, L.kmask, nullptr, nullptr, n, colour, h2inv, (T)c.nu, (T)c.kap, sp,
-                    (T)(sqDf * sqDf), lsn, L.lamp, etanu);
+                    (T)(sqDf * sqDf), lsn, L.lamp, T(0));
+            }
             ctx->end();
         }
     }
@@ -1438,33 +1484,47 @@ static int residual(Exec* ctx, Level<T>& L, const T* u, const T* F, T fscale, T 
         }
     }
     if constexpr (sizeof(T) == 8) {
-        // FP64 levels from 64^3 up without a background: the z-marching kernel
-        if (!L.bg && !L.gap && n >= 64) {
-            int nz = 8;
+        // FP64 levels (they have no background): cell64.cuh
+        const K64 k = make_k64(n, c.nu, c.kap, c.eta);
+        const double Dfl = L.fine ? k.Df : 0.0;
+        ctx->begin(PM_K_RESID64, L.fine, (long long)L.cells);
+        if (n >= 64) {
+            // few planes per block on 64^3, so that every SM has one (256 blocks)
+            int nz = n == 64 ? 4 : 8;
             while ((size_t)(n / kR64TX) * (n / kR64TY) * (n / nz) > (size_t)kMaxPartials) nz *= 2;
             const dim3 g3(n / kR64TX, n / kR64TY, n / nz);
-            ctx->begin(PM_K_RESID64, L.fine, (long long)L.cells);
-            k_residual64_zm<WRITE_R, MIXED><<<g3, 256, 0, ctx->stream>>>(
-                u, F, fscale, lam, L.kmask, n, nz, h2inv, c.nu, c.kap, sqDf * sqDf, (double)lsn, L.fine, L.r, L.sat,
-                ctx->red_partials, rplain, chi32, gap32, L.lamp, ctx->red_out);
-            ctx->end();
-            return (int)(g3.x * g3.y * g3.z);
+            grid = (int)(g3.x * g3.y * g3.z);
+            if (L.kmask)
+                k_residual64_zm<WRITE_R, MIXED, true><<<g3, 256, 0, ctx->stream>>>(
+                    u, F, fscale, lam, L.kmask, n, nz, k, Dfl, L.r, L.sat, ctx->red_partials, rplain, chi32, gap32,
+                    L.lamp, ctx->red_out);
+            else
+                k_residual64_zm<WRITE_R, MIXED, false><<<g3, 256, 0, ctx->stream>>>(
+                    u, F, fscale, lam, nullptr, n, nz, k, Dfl, L.r, L.sat, ctx->red_partials, rplain, chi32, gap32,
+                    L.lamp, ctx->red_out);
+        } else {
+            const int th = std::max(64, thin_threads(ctx, L.cells));
+            grid = (int)((L.cells + th - 1) / th);
+            k_residual64<<<grid, th, 0, ctx->stream>>>(u, F, fscale, lam, L.kmask, n, __builtin_ctz(n), k, Dfl,
+                                                       WRITE_R ? L.r : nullptr, WRITE_R ? L.sat : nullptr,
+                                                       ctx->red_partials, MIXED ? rplain : nullptr, chi32, gap32,
+                                                       L.lamp, ctx->red_out);
         }
-    }
-    if (L.bg) {
-        ctx->begin(sizeof(T) == 8 ? PM_K_RESID64 : PM_K_RESID32, L.fine, (long long)L.cells);
-        k_residual<T, true, WRITE_R, MIXED><<<grid, kThreads, 0, ctx->stream>>>(
-            u, F, fscale, lam, L.kmask, L.bg, L.gap, n, h2inv, (T)c.nu, (T)c.kap, (T)(sqDf * sqDf), lsn, L.fine, L.r,
-            L.sat, ctx->red_partials, rplain, chi32, gap32, L.lamp, ctx->red_out);
         ctx->end();
+        return grid;
     } else {
-        ctx->begin(sizeof(T) == 8 ? PM_K_RESID64 : PM_K_RESID32, L.fine, (long long)L.cells);
-        k_residual<T, false, WRITE_R, MIXED><<<grid, kThreads, 0, ctx->stream>>>(
-            u, F, fscale, lam, L.kmask, nullptr, nullptr, n, h2inv, (T)c.nu, (T)c.kap, (T)(sqDf * sqDf), lsn, L.fine,
-            L.r, L.sat, ctx->red_partials, rplain, chi32, gap32, L.lamp, ctx->red_out);
+        ctx->begin(PM_K_RESID32, L.fine, (long long)L.cells);
+        if (L.bg)
+            k_residual<T, true, WRITE_R, MIXED><<<grid, kThreads, 0, ctx->stream>>>(
+                u, F, fscale, lam, L.kmask, L.bg, L.gap, n, h2inv, (T)c.nu, (T)c.kap, (T)(sqDf * sqDf), lsn, L.fine,
+                L.r, L.sat, ctx->red_partials, rplain, chi32, gap32, L.lamp, ctx->red_out);
+        else
+            k_residual<T, false, WRITE_R, MIXED><<<grid, kThreads, 0, ctx->stream>>>(
+                u, F, fscale, lam, L.kmask, nullptr, nullptr, n, h2inv, (T)c.nu, (T)c.kap, (T)(sqDf * sqDf), lsn,
+                L.fine, L.r, L.sat, ctx->red_partials, rplain, chi32, gap32, L.lamp, ctx->red_out);
         ctx->end();
+        return grid;
     }
-    return grid;
 }
 
 // The residual of a large FP32 level with the FAS restriction to C folded in
@@ -1516,14 +1576,15 @@ static void level_down(Exec* ctx, std::vector<Level<T>>& lv, int l, const T* F0,
     for (int s = 0; s < ctx->prm.npre; ++s) sweep(ctx, L, F, fs, lam, c);
     Level<T>& C = lv[l + 1];
     C.cur = 0;
-    const int gc = grid_for(ctx, C.cells);
+    const int th = sizeof(T) == 8 ? thin_threads(ctx, C.cells) : kThreads;
+    const int gc = grid_for(ctx, C.cells, th);
     // large FP32 levels: the residual kernel restricts as well (gauge term left to k_fas_rhs)
     bool fused = false;
     if constexpr (sizeof(T) == 4) fused = residual_restrict_f32(ctx, L, C, L.u[L.cur], F, fs, lam, c);
     if (!fused) {
         residual<T, true, false>(ctx, L, L.u[L.cur], F, fs, lam, c, nullptr, nullptr);
         ctx->begin(PM_K_TRANSFER, false, 0);
-        k_restrict_fas<T><<<gc, kThreads, 0, ctx->stream>>>(L.u[L.cur], L.r, L.sat, L.kmask, ctx->red_out + 8, C.n,
+        k_restrict_fas<T><<<gc, th, 0, ctx->stream>>>(L.u[L.cur], L.r, L.sat, L.kmask, ctx->red_out + 8, C.n,
                                                             C.ur, C.u[0], C.r, C.kmask);
         ctx->end();
     }
@@ -1546,10 +1607,12 @@ static void level_down(Exec* ctx, std::vector<Level<T>>& lv, int l, const T* F0,
         ctx->begin(PM_K_TRANSFER, false, 0);
         if (C.n >= 32)
             k_fas_rhs_tile<T, false><<<dim3(C.n / 32, C.n / 4, C.n / 4), 256, 0, ctx->stream>>>(
-                C.u[0], C.r, C.kmask, nullptr, C.n, ih2c, (T)c.nu, (T)c.kap, C.f, nullptr, nullptr, 0.f, gmp);
+                C.u[0], C.r, C.kmask, nullptr, C.n, ih2c, (T)c.nu, (T)c.kap, C.f, nullptr, nullptr, 0.f, gmp,
+                make_k64(C.n, c.nu, c.kap, c.eta));
         else
-            k_fas_rhs<T, false><<<gc, kThreads, 0, ctx->stream>>>(C.u[0], C.r, C.kmask, nullptr, C.n, ih2c, (T)c.nu,
-                                                                  (T)c.kap, C.f, nullptr, nullptr, 0.f, gmp);
+            k_fas_rhs<T, false><<<gc, th, 0, ctx->stream>>>(C.u[0], C.r, C.kmask, nullptr, C.n, ih2c, (T)c.nu,
+                                                            (T)c.kap, C.f, nullptr, nullptr, 0.f, gmp,
+                                                            make_k64(C.n, c.nu, c.kap, c.eta));
         ctx->end();
     }
 }
@@ -1567,8 +1630,10 @@ static void level_up(Exec* ctx, std::vector<Level<T>>& lv, int l, const T* F0, T
     if (C.n >= 32)
         k_prolong_add_tile<T><<<dim3(C.n / 32, C.n / 4, C.n / 4), 256, 0, ctx->stream>>>(C.u[C.cur], C.ur, C.n,
                                                                                           L.u[L.cur]);
-    else
-        k_prolong_add<T><<<grid_for(ctx, C.cells), kThreads, 0, ctx->stream>>>(C.u[C.cur], C.ur, C.n, L.u[L.cur]);
+    else {
+        const int th = sizeof(T) == 8 ? thin_threads(ctx, C.cells) : kThreads;
+        k_prolong_add<T><<<grid_for(ctx, C.cells, th), th, 0, ctx->stream>>>(C.u[C.cur], C.ur, C.n, L.u[L.cur]);
+    }
     ctx->end();
     for (int s = 0; s < ctx->prm.npost; ++s) sweep(ctx, L, F, fs, lam, c);
 }
@@ -1597,12 +1662,13 @@ static void vcycle(Exec* ctx, std::vector<Level<T>>& lv, int l, const T* F0, T f
         if (L.bg) {
             ctx->begin(PM_K_COARSEST, false, 0);
             k_coarsest<T, true><<<1, 256, 0, ctx->stream>>>(L.u[L.cur], F, fs, L.kmask, L.bg, L.n, ih2, c.nu, c.kap,
-                                                            c.eta, ctx->prm.coarse_sweeps, L.fine);
+                                                            c.eta, ctx->prm.coarse_sweeps, L.fine, K64{});
             ctx->end();
         } else {
             ctx->begin(PM_K_COARSEST, false, 0);
             k_coarsest<T, false><<<1, 256, 0, ctx->stream>>>(L.u[L.cur], F, fs, L.kmask, nullptr, L.n, ih2, c.nu,
-                                                             c.kap, c.eta, ctx->prm.coarse_sweeps, L.fine);
+                                                             c.kap, c.eta, ctx->prm.coarse_sweeps, L.fine,
+                                                             make_k64(L.n, c.nu, c.kap, c.eta));
             ctx->end();
         }
         return;
