@@ -10,9 +10,10 @@
 // Forward (implicit GEMM): M = voxels (128 per block), N = Cout, K = 27 x Cin, streamed in
 // steps of one tap x 16 channels with a two-stage cp.async pipeline.  The backward data
 // pass is the same kernel with the weights flipped in space and transposed in channels,
-// followed by the ReLU mask of the layer input.  The weight gradient is a GEMM over voxels
-// per tap: each block owns one tap and a chunk of voxels, stages both operands transposed
-// in shared memory (channels x voxels) and writes an FP32 partial reduced in fixed order.
+// followed by the ReLU mask of the layer input.  The weight gradient of levels below 16^3 is a
+// GEMM over voxels per tap: each block owns one tap and a chunk of voxels, stages both operands
+// transposed in shared memory (channels x voxels) and writes an FP32 partial reduced in fixed
+// order; larger levels take wgrad.cuh.
 #pragma once
 
 #include <cuda_bf16.h>

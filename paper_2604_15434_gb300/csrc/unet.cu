@@ -21,6 +21,7 @@
 #include "conv.cuh"
 #include "conv_umma.cuh"
 #include "internal.cuh"
+#include "wgrad.cuh"
 
 struct pm_unet;
 
@@ -203,16 +204,6 @@ __global__ void k_bias_grad(const __nv_bfloat16* __restrict__ dy, int ld, int of
     }
 }
 
-// grad[i] += sum over blocks of partials[b][i] (fixed order)
-__global__ void k_reduce_add(const float* __restrict__ partials, int nblocks, int count, float* __restrict__ grad)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * count + i];
-        grad[i] += s;
-    }
-}
-
 // Adam on the flat FP32 parameters, then zero the gradient accumulator
 __global__ void k_adam(float* __restrict__ p, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                        long long count, float lr, float b1, float b2, float eps, float c1, float c2)
@@ -312,6 +303,9 @@ static void free_acts(Acts& a)
     a = Acts();
 }
 
+// the weight gradient's partial sums (chunks) for an n^3 level
+static int wgrad_rows(int n) { return (int)(((size_t)n * n * n + kWgChunk - 1) / kWgChunk); }
+
 static pm_status ensure_acts(pm_unet* u, int n, bool train)
 {
     pm_ctx* ctx = u->ctx;
@@ -347,12 +341,11 @@ static pm_status ensure_acts(pm_unet* u, int n, bool train)
         PM_TRY(dalloc(ctx, &a.d2, v1 * 32));
         PM_TRY(dalloc(ctx, &a.dp1, v1 * 16));
         PM_TRY(dalloc(ctx, &a.d0, v0 * 16));
-        // largest partial buffer: chunks * 27 * ci * co over the convs
+        // largest partial buffer over the convs: their weight partials, then the bias rows
         size_t mx = 0;
         for (int i = 0; i < 10; ++i) {
-            const size_t nv = (size_t)(n >> kConvs[i].level) * (n >> kConvs[i].level) * (n >> kConvs[i].level);
-            const size_t chunks = (nv + 8191) / 8192;
-            mx = std::max(mx, chunks * 27 * kConvs[i].ci * kConvs[i].co);
+            const int nl = n >> kConvs[i].level, rows = wgrad_rows(nl);
+            mx = std::max(mx, (size_t)rows * (27 * kConvs[i].ci + 1) * kConvs[i].co);
         }
         mx = std::max(mx, (size_t)kMaxPartials * 96);
         a.part_count = mx;
@@ -494,38 +487,56 @@ static void conv_fwd(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off
     ctx->end();
 }
 
-// weight gradient of conv i: grad[off .. off + 27 ci co) += sum over voxels; then the bias
+template <int CO, int KX>
+static void launch_wgrad(pm_ctx* ctx, const __nv_bfloat16* x, int x_ld, int x_off, const __nv_bfloat16* dy, int dy_ld,
+                         int dy_off, int n, int ci, int co, int rows, float* part, float* bpart)
+{
+    const size_t smem = wgrad_smem(n, CO, KX);
+    cudaFuncSetAttribute(k_wgrad<CO, KX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_wgrad<CO, KX><<<dim3(rows, (ci / 16) * (3 / KX), co / CO), kWgThreads, smem, ctx->stream>>>(
+        x, x_ld, x_off, dy, dy_ld, dy_off, n, ci, co, part, bpart);
+}
+
+// weight and bias gradient of conv i: grad[off ..] += sums over the voxels.  Levels of at least
+// 16^3 take the staged kernel (wgrad.cuh), smaller ones the per-tap kernel.
 static void conv_wgrad(pm_unet* u, int i, const __nv_bfloat16* x, int x_ld, int x_off, const __nv_bfloat16* dy,
                        int dy_ld, int dy_off, int n)
 {
     pm_ctx* ctx = u->ctx;
     const int ci = kConvs[i].ci, co = kConvs[i].co;
-    const int nvox = n * n * n;
-    const int chunk = 8192, chunks = (nvox + chunk - 1) / chunk;
-    const dim3 grid(27, chunks);
+    const int nvox = n * n * n, count = 27 * ci * co, rows = wgrad_rows(n);
+    float* bpart = u->acts.part + (size_t)rows * count;
+    int brows = rows;
     ctx->begin(PM_K_PM);
+    if (n >= kWgMin) {
+        // blocks of all taps and up to 32 outputs where that makes at least one per SM, else of one z
+        // tap and 16 outputs (six times the blocks at 32 outputs)
+        const auto launch = co % 32 != 0 ? ((long long)rows * (ci / 16) >= ctx->num_sms ? launch_wgrad<16, 3> : launch_wgrad<16, 1>)
+                                         : ((long long)rows * (ci / 16) * (co / 32) >= ctx->num_sms ? launch_wgrad<32, 3> : launch_wgrad<16, 1>);
+        launch(ctx, x, x_ld, x_off, dy, dy_ld, dy_off, n, ci, co, rows, u->acts.part, bpart);
+        ctx->end();
+    } else {
+        const dim3 grid(27, rows);
 #define PM_WG_CASE(CI_, CO_)                                                                                        \
     if (ci == CI_ && co == CO_)                                                                                     \
-        k_conv3d_wgrad<CI_, CO_><<<grid, 128, 0, ctx->stream>>>(x, x_ld, x_off, dy, dy_ld, dy_off, n, chunk, u->acts.part);
-    PM_WG_CASE(16, 16)
-    PM_WG_CASE(16, 32)
-    PM_WG_CASE(32, 32)
-    PM_WG_CASE(32, 64)
-    PM_WG_CASE(64, 64)
-    PM_WG_CASE(96, 32)
-    PM_WG_CASE(48, 16)
+        k_conv3d_wgrad<CI_, CO_><<<grid, 128, 0, ctx->stream>>>(x, x_ld, x_off, dy, dy_ld, dy_off, n, kWgChunk, u->acts.part);
+        PM_WG_CASE(16, 32)
+        PM_WG_CASE(32, 32)
+        PM_WG_CASE(32, 64)
+        PM_WG_CASE(64, 64)
+        PM_WG_CASE(96, 32)
 #undef PM_WG_CASE
-    ctx->end();
-    const int count = 27 * ci * co;
+        ctx->end();
+        brows = 1;  // at most 512 voxels
+        ctx->begin(PM_K_PM);
+        k_bias_grad<<<brows, 256, 0, ctx->stream>>>(dy, dy_ld, dy_off, co, nvox, bpart);
+        ctx->end();
+    }
     ctx->begin(PM_K_PM);
-    k_reduce_add<<<blocks_for(ctx, count), 256, 0, ctx->stream>>>(u->acts.part, chunks, count, u->g + u->off[i]);
-    ctx->end();
-    const int bb = std::min(blocks_for(ctx, nvox), kMaxPartials);
-    ctx->begin(PM_K_PM);
-    k_bias_grad<<<bb, 256, 0, ctx->stream>>>(dy, dy_ld, dy_off, co, nvox, u->acts.part);
+    k_sum_rows_add<<<(count + 31) / 32, 256, 0, ctx->stream>>>(u->acts.part, rows, count, u->g + u->off[i]);
     ctx->end();
     ctx->begin(PM_K_PM);
-    k_reduce_add<<<1, 256, 0, ctx->stream>>>(u->acts.part, bb, co, u->g + u->off[i] + 27LL * ci * co);
+    k_sum_rows_add<<<(co + 31) / 32, 256, 0, ctx->stream>>>(bpart, brows, co, u->g + u->off[i] + count);
     ctx->end();
 }
 
