@@ -208,83 +208,120 @@ __global__ void k_f2d(const float* __restrict__ x, size_t total, double* __restr
         y[c] = (double)x[c];
 }
 
-// Psi = psiN + xi chi on the grid (psiN alone when chi is null), rounded as written.
-__global__ void k_psi_total(const double* __restrict__ psiN, const double* __restrict__ chi, double xi,
-                            size_t total, double* __restrict__ psi)
+// Psi = psiN + xi chi on the grid, rounded as written.
+__global__ void __launch_bounds__(256) k_psi_total(const double* __restrict__ psiN, const double* __restrict__ chi,
+                                                   double xi, size_t total, double* __restrict__ psi)
 {
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x)
-        psi[c] = chi ? __dadd_rn(psiN[c], __dmul_rn(xi, chi[c])) : psiN[c];
+        psi[c] = __dadd_rn(psiN[c], __dmul_rn(xi, chi[c]));
 }
 
-// g = -grad Psi on the grid, one cell per thread: the five-point difference
-// (-f+2 + 8 f+1 - 8 f-1 + f-2)/(12 h) per axis (FOUR; else the two-point (f+1 - f-1)/(2 h)),
-// periodic.  g holds the three components one after the other ([3][n^3]).
+// The grid force up to its scale: G = 8 (f+1 - f-1) - (f+2 - f-2) per axis (FOUR; else f+1 - f-1) of
+// the potential, periodic, one cell per thread; -grad Psi is G times -n/12 (-n/2), a factor the
+// interpolation applies.  g holds (Gx, Gy, Gz, 0) per cell, 32 bytes, so that a particle's corner
+// is one aligned 256-bit load.  Bound by FP64 instructions: three per component where the scaled
+// difference took four (0.40 -> 0.295 ms at 256^3).  (A z-marching block that formed Psi itself
+// recomputed it on its halo, 2.9 instructions per cell instead of 2: 0.43 ms against 0.37 for the
+// two kernels.)
 template <bool FOUR>
-__global__ void __launch_bounds__(256) k_grad(const double* __restrict__ psi, int n, double* __restrict__ g)
+__global__ void __launch_bounds__(256) k_grad(const double* __restrict__ psi, int n, int lg, double* __restrict__ g)
 {
     const int m = n - 1;
     const size_t total = (size_t)n * n * n;
-    const double inv12h = (double)n / 12.0, inv2h = (double)n * 0.5;
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(c & (size_t)m);  // n is a power of two
-        const int j = (int)((c / n) & (size_t)m), k = (int)(c / ((size_t)n * n));
-        auto at = [&](int x, int y, int z) { return psi[((size_t)(z & m) * n + (y & m)) * n + (x & m)]; };
-        double gx, gy, gz;
+        const int i = (int)(c & (size_t)m), j = (int)((c >> lg) & (size_t)m), k = (int)(c >> (2 * lg));
+        const double* row = psi + (c - i);
+        const double* col = psi + (((size_t)k << (2 * lg)) + i);
+        const double* pil = psi + (((size_t)j << lg) + i);
+        auto x = [&](int d) { return row[(i + d) & m]; };
+        auto y = [&](int d) { return col[(size_t)((j + d) & m) << lg]; };
+        auto z = [&](int d) { return pil[(size_t)((k + d) & m) << (2 * lg)]; };
+        double gx = x(1) - x(-1), gy = y(1) - y(-1), gz = z(1) - z(-1);
         if (FOUR) {
-            gx = (-at(i + 2, j, k) + 8.0 * at(i + 1, j, k) - 8.0 * at(i - 1, j, k) + at(i - 2, j, k)) * inv12h;
-            gy = (-at(i, j + 2, k) + 8.0 * at(i, j + 1, k) - 8.0 * at(i, j - 1, k) + at(i, j - 2, k)) * inv12h;
-            gz = (-at(i, j, k + 2) + 8.0 * at(i, j, k + 1) - 8.0 * at(i, j, k - 1) + at(i, j, k - 2)) * inv12h;
-        } else {
-            gx = (at(i + 1, j, k) - at(i - 1, j, k)) * inv2h;
-            gy = (at(i, j + 1, k) - at(i, j - 1, k)) * inv2h;
-            gz = (at(i, j, k + 1) - at(i, j, k - 1)) * inv2h;
+            gx = fma(8.0, gx, x(-2) - x(2));
+            gy = fma(8.0, gy, y(-2) - y(2));
+            gz = fma(8.0, gz, z(-2) - z(2));
         }
-        g[c] = -gx;
-        g[total + c] = -gy;
-        g[2 * total + c] = -gz;
+        double2* o = reinterpret_cast<double2*>(g + 4 * c);
+        o[0] = make_double2(gx, gy);
+        o[1] = make_double2(gz, 0.0);
     }
 }
 
-// the force at each particle: the grid force g ([3][n^3]) at the 8 CIC corners (in the
-// deposit's corner order), weighted by the corner's CIC weight (the deposit's adjoint)
-__global__ void __launch_bounds__(256) k_interp_force(const double* __restrict__ g, int n,
+// f 2^-63 as a double (correctly rounded but for exact ties), f <= 2^63: the integer pipe's conversion
+__device__ __forceinline__ double fixed_to_double(unsigned long long f)
+{
+    if (f == 0) return 0.0;
+    const int lz = __clzll((long long)f);
+    const unsigned long long m = f << lz;  // top bit set
+    return __longlong_as_double((long long)(((unsigned long long)(1022 - lz) << 52) + (m >> 11) + ((m >> 10) & 1)));
+}
+
+// four doubles of one 32-byte aligned cell
+__device__ __forceinline__ void ld_cell(const double* p, double& a, double& b, double& c)
+{
+    double unused;
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(unused) : "l"(p));
+}
+
+// The force at each particle: the grid force at the 8 CIC corners weighted by the corners' CIC
+// weights (the deposit's adjoint), times `scale`.  Bound by FP64 instructions (39 per particle where
+// eight weights, three-component sums and the weights' floors and conversions took 54): the weights
+// come from the integer pipe, the x-y weights serve both z planes, and the scale rides on the z
+// weights.  256^3 particles: 1.64 -> 1.19 ms.
+__global__ void __launch_bounds__(256) k_interp_force(const double* __restrict__ g, int n, double scale,
                                                       const double* __restrict__ pos, long long np,
                                                       double* __restrict__ acc)
 {
-    const int m = n - 1;
-    const size_t total = (size_t)n * n * n;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (long long)gridDim.x * blockDim.x) {
-        int ix[2], iy[2], iz[2];
-        double wx[2], wy[2], wz[2];
-        cic_1d(pos[p], n, ix[0], ix[1], wx[0], wx[1]);
-        cic_1d(pos[np + p], n, iy[0], iy[1], wy[0], wy[1]);
-        cic_1d(pos[2 * np + p], n, iz[0], iz[1], wz[0], wz[1]);
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int a = c & 1, b = (c >> 1) & 1, e = (c >> 2) & 1;
-            const size_t cell = ((size_t)(iz[e] & m) * n + (iy[b] & m)) * n + (ix[a] & m);
-            const double w = __dmul_rn(__dmul_rn(wx[a], wy[b]), wz[e]);
-            s0 += w * g[cell];
-            s1 += w * g[total + cell];
-            s2 += w * g[2 * total + cell];
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= np) return;
+    int ix[2], iy[2], iz[2];
+    double wx[2], wy[2], wz[2];
+    auto axis = [&](double x, int (&i)[2], double (&w)[2]) {
+        const CicFixed f = cic_fixed(x, n);
+        if (f.ok) {
+            i[0] = f.i0;
+            i[1] = f.i1;
+            w[0] = fixed_to_double(f.w0);
+            w[1] = fixed_to_double(f.w1);
+        } else {
+            cic_1d(x, n, i[0], i[1], w[0], w[1]);
         }
-        acc[p] = s0;
-        acc[np + p] = s1;
-        acc[2 * np + p] = s2;
-    }
+    };
+    axis(pos[p], ix, wx);
+    axis(pos[np + p], iy, wy);
+    axis(pos[2 * np + p], iz, wz);
+    double s[2][3];
+    const double w4[4] = {wx[0] * wy[0], wx[1] * wy[0], wx[0] * wy[1], wx[1] * wy[1]};
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            double a, b, d;
+            ld_cell(g + 4 * (((size_t)iz[e] * n + iy[c >> 1]) * n + ix[c & 1]), a, b, d);
+            s[e][0] = c ? fma(w4[c], a, s[e][0]) : w4[c] * a;
+            s[e][1] = c ? fma(w4[c], b, s[e][1]) : w4[c] * b;
+            s[e][2] = c ? fma(w4[c], d, s[e][2]) : w4[c] * d;
+        }
+    const double z0 = wz[0] * scale, z1 = wz[1] * scale;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) acc[k * np + p] = fma(z1, s[1][k], z0 * s[0][k]);
 }
 
-// v += g dt; x = frac(x + v dt), each product and sum rounded as written.
-__global__ void k_kick_drift(double* __restrict__ pos, double* __restrict__ vel, const double* __restrict__ acc,
-                             long long total, double dt)
+// v += g dt; x = frac(x + v dt), each product and sum rounded as written.  FP64 instructions bound
+// it (four per coordinate): the wrap is entered only where the bits of x say x < 0 or x >= 1
+// (50 M coordinates: 0.68 -> 0.42 ms).
+__global__ void __launch_bounds__(256) k_kick_drift(double* __restrict__ pos, double* __restrict__ vel,
+                                                    const double* __restrict__ acc, long long total, double dt)
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const double v = __dadd_rn(vel[i], __dmul_rn(acc[i], dt));
         vel[i] = v;
         double x = __dadd_rn(pos[i], __dmul_rn(v, dt));
-        x = __dsub_rn(x, floor(x));
-        if (x >= 1.0) x = 0.0;
+        if ((unsigned)__double2hiint(x) >= 0x3ff00000u) {  // negative, >= 1 or not a number
+            x = __dsub_rn(x, floor(x));
+            if (x >= 1.0) x = 0.0;
+        }
         pos[i] = x;
     }
 }
@@ -398,8 +435,8 @@ pm_status poisson32(pm_ctx* ctx, const double* delta, int n, double fac, double*
     return PM_OK;
 }
 
-// g = -grad(psiN + xi chi) at each particle (Eq. force, Sec. 3.5.2): the total potential and
-// its gradient on the grid (workspace [4][n^3]: Psi, then the three components), then the
+// g = -grad(psiN + xi chi) at each particle (Eq. force, Sec. 3.5.2; psiN alone when chi is null): the
+// total potential and its gradient on the grid (workspace: [n^3][4] force, then [n^3] Psi), then the
 // CIC interpolation of the grid force.
 pm_status interp_force(pm_ctx* ctx, const double* psiN, const double* chi, double xi, int n, const double* pos,
                        long long np, double* acc)
@@ -407,20 +444,24 @@ pm_status interp_force(pm_ctx* ctx, const double* psiN, const double* chi, doubl
     Workspace* w = nullptr;
     PM_TRY(get_workspace(ctx, n, &w));
     const size_t cells = (size_t)n * n * n;
-    if (!w->grad) PM_CUDA(cudaMalloc(&w->grad, 4 * cells * sizeof(double)));
-    double* psi = w->grad;
-    double* g = w->grad + cells;
+    if (!w->grad) PM_CUDA(cudaMalloc(&w->grad, 5 * cells * sizeof(double)));
+    const double* psi = psiN;
+    if (chi) {
+        double* sum = w->grad + 4 * cells;
+        ctx->begin(PM_K_PM, false, 0);
+        k_psi_total<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psiN, chi, xi, cells, sum);
+        ctx->end();
+        psi = sum;
+    }
+    const bool four = ctx->prm.grad_order != 2;
+    const int lg = __builtin_ctz(n);
     ctx->begin(PM_K_PM, false, 0);
-    k_psi_total<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psiN, chi, xi, cells, psi);
+    if (four) k_grad<true><<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psi, n, lg, w->grad);
+    else k_grad<false><<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psi, n, lg, w->grad);
     ctx->end();
     ctx->begin(PM_K_PM, false, 0);
-    if (ctx->prm.grad_order == 2)
-        k_grad<false><<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psi, n, g);
-    else
-        k_grad<true><<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psi, n, g);
-    ctx->end();
-    ctx->begin(PM_K_PM, false, 0);
-    k_interp_force<<<grid_for(ctx, (size_t)np), kThreads, 0, ctx->stream>>>(g, n, pos, np, acc);
+    k_interp_force<<<(unsigned)((np + kThreads - 1) / kThreads), kThreads, 0, ctx->stream>>>(
+        w->grad, n, four ? -(double)n / 12.0 : -(double)n * 0.5, pos, np, acc);
     ctx->end();
     PM_CUDA(cudaGetLastError());
     return PM_OK;

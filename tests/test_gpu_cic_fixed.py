@@ -4,6 +4,7 @@ product can round either way, and the force at the same particles against its pl
 Positions: cell centres and faces and their neighbours in FP64 (weights 0, 1 and within one ulp of
 them), the first half cell (s < 0) and the first cell (s < 1, inexact weights), dyadic fractions whose
 weight products sit on exact ties of 2^-40, coordinates outside [0, 1), and random ones.
+Force tolerance: 24 products and sums of 2^-53 each of the largest corner value: 1e-14 of it.
 """
 import numpy as np
 import pytest
@@ -39,3 +40,16 @@ def test_density_with_a_power_of_two_mean(gpu_lib):
         got = gpu_lib.pm_deposit_cic(torch.from_numpy(pos).cuda(), n).cpu().numpy()
         assert np.array_equal(got, O.density(O.deposit_cic(pos, n), count))
 
+
+@pytest.mark.parametrize("n,count", [(8, 1), (16, 777), (64, 50001)])
+@pytest.mark.parametrize("order", [4, 2])
+def test_force(gpu_lib, n, count, order):
+    rng = np.random.default_rng(n + order)
+    psi, chi = rng.standard_normal((2, n, n, n))
+    pos = positions(n, count, 5 * n)
+    ctx = gpu_lib.Context(grad_order=order)
+    got = gpu_lib.force_interp(torch.from_numpy(psi).cuda(), torch.from_numpy(chi).cuda(), -1.0, 0.2, 1.0,
+                               torch.from_numpy(pos).cuda(), ctx=ctx).cpu().numpy()
+    g = O.accel_grid(psi, chi, gpu_lib.coefficients(-1.0, 0.2, 1.0)["xi"], n, order=order)
+    want = O.interp_cic(g, pos)
+    assert np.abs(got - want).max() <= 1e-14 * np.abs(g).max()
