@@ -70,9 +70,11 @@ typedef struct {
     int grad_order;        /* force_interp / pm_step gradient: 4 the five-point fourth-order difference of
                               Sec. 3.5.2, 2 the two-point central difference (4) */
     int batch_persistent;  /* scalar_mg_solve_batched: 1 runs the inner V-cycle's levels 32^3 .. 4^3 of every box of
-                              at least 64^3 in one persistent cooperative launch per outer iteration, with grid
-                              barriers whose waits are bounded (PM_ERR_TIMEOUT when one gives up); 0 launches
-                              them per box (1; applies with coarse_exact = 0, coarsest_n = 4, inner_cycles = 1) */
+                              at least 64^3 in one launch per box (a thread-block cluster, as in scalar_mg_solve),
+                              or, where the device cannot hold that cluster, in one persistent cooperative launch
+                              of all boxes per outer iteration, with grid barriers whose waits are bounded
+                              (PM_ERR_TIMEOUT when one gives up); 0 launches them level by level (1; applies with
+                              coarse_exact = 0, coarsest_n = 4, the cooperative launch with inner_cycles = 1) */
     int zero_start;        /* precision 1: the first sweep of each inner cycle on the finest inner level of grids
                               >= 256^3 (the level that receives the background's coefficients) runs the
                               zero-start kernel, which exploits that the correction starts at zero (same
@@ -167,7 +169,7 @@ pm_status scalar_mg_solve_batched(pm_ctx* ctx, int nbox, const int* n, const dou
 
 /*
  * Test hook of the batched solve's bounded grid barrier (pm_params.batch_persistent).  With
- * block >= 0, block `block` of the persistent coarse-level kernel leaves the kernel just
+ * block >= 0 the batched solve takes the cooperative launch whether or not the cluster fits, and block `block` of the persistent coarse-level kernel leaves the kernel just
  * before its `barrier`-th grid barrier (counted from 0) in every launch, so that the other
  * blocks' bounded waits run out: the batched solve then returns PM_ERR_TIMEOUT with its
  * results undefined, and the context stays usable.  Nothing faults: the blocks only stop

@@ -34,6 +34,8 @@ struct BoxRun {
     int cyc = 0, vcyc = 0;
     pm_status st = PM_ERR_NOCONV;
     bool active = false, trivial = false;
+    bool cluster = false;  // the coarse inner levels in one cluster launch of its own (coarse_cluster.cuh)
+    const int* cluster_active = nullptr;
     size_t cells = 0;
     double hist[64] = {};
     double guess_rr = 0.0;
@@ -41,6 +43,15 @@ struct BoxRun {
     FFCoef fk{};
     double lam_fix = 0.0;  // gauge shift found by the confirming FP64 residual
 };
+
+// where the box's work goes: its own stream and reduction buffers
+static Exec box_exec(pm_ctx* ctx, const BoxRun& B)
+{
+    Exec x(ctx, B.w->stream, B.w->partials, B.w->out, B.w->host, false);
+    x.cluster = B.cluster;
+    x.cluster_active = B.cluster_active;
+    return x;
+}
 
 static pm_status box_prepare(pm_ctx* ctx, Workspace* w)
 {
@@ -74,11 +85,7 @@ static void box_iteration(Exec* x, BoxRun& B)
 {
     Workspace* w = B.w;
     auto& s = w->s;
-    for (size_t l = 0; l + 1 < s.size(); ++l) {
-        x->begin(PM_K_TRANSFER);
-        k_restrict<float><<<grid_for(x, s[l + 1].cells), kThreads, 0, x->stream>>>(s[l].bg, s[l + 1].n, s[l + 1].bg);
-        x->end();
-    }
+    restrict_background(x, s);
     s[0].lamp = w->shift;
     start_at_zero(x, s[0]);
     for (int k = 0; k < x->prm.inner_cycles; ++k) vcycle<float>(x, s, 0, w->rplain, 1.0f, 0.0f, B.c);
@@ -94,11 +101,7 @@ static void box_down(Exec* x, BoxRun& B, int l32)
 {
     Workspace* w = B.w;
     auto& s = w->s;
-    for (size_t l = 0; l + 1 < s.size(); ++l) {
-        x->begin(PM_K_TRANSFER);
-        k_restrict<float><<<grid_for(x, s[l + 1].cells), kThreads, 0, x->stream>>>(s[l].bg, s[l + 1].n, s[l + 1].bg);
-        x->end();
-    }
+    restrict_background(x, s);
     s[0].lamp = w->shift;
     start_at_zero(x, s[0]);
     vcycle_down<float>(x, s, l32, w->rplain, 1.0f, 0.0f, B.c);
@@ -226,7 +229,11 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
         PM_TRY(ensure_mg(ctx, w, true));
         PM_TRY(box_prepare(ctx, w));
         PM_CUDA(cudaStreamWaitEvent(w->stream, ready, 0));
-        Exec x(ctx, w->stream, w->partials, w->out, w->host, false);
+        // the coarse levels: a cluster launch per box, which runs beside the other boxes' kernels, or,
+        // where the cluster does not fit the device (and for the barrier's test hook), the cooperative
+        // kernel of all boxes, which holds every box up (24 boxes: 0.56 ms per iteration)
+        Exec x = box_exec(ctx, R);
+        R.cluster = x.cluster = P.batch_persistent && ctx->coop_fail_block < 0 && cluster_levels(&x, w->s);
         PM_TRY(source_norm(&x, R.delta, R.cells, R.cf.src, &R.fnorm));
         w->d[0].cur = 0;
         R.fk = make_ffcoef(R.cf.nu, R.cf.kappa, P.eta, nn[b]);
@@ -255,7 +262,7 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
             R.guess_rejected = true;
             R.st = PM_ERR_NOCONV;
             R.active = true;
-            Exec x(ctx, R.w->stream, R.w->partials, R.w->out, R.w->host, false);
+            Exec x = box_exec(ctx, R);
             PM_CUDA(cudaMemsetAsync(ff_chi(R.w), 0, R.cells * sizeof(float2), R.w->stream));
             PM_CUDA(cudaMemsetAsync(R.w->lam, 0, sizeof(double), R.w->stream));
             box_residual(&x, R);
@@ -268,10 +275,23 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                 PM_CUDA(cudaStreamSynchronize(B[b].w->stream));
                 box_check(P, B[b], tol);
             }
+    // flags of the boxes whose coarse levels are cluster launches (these and the cooperative boxes share
+    // one array: either form serves all boxes of a call)
+    std::vector<int> cluster_idx(nbox, -1);
+    int ncluster = 0;
+    for (int b = 0; b < nbox; ++b)
+        if (B[b].active && B[b].cluster) cluster_idx[b] = ncluster++;
+    if (ncluster > 0) {
+        PM_TRY(coop_alloc(ctx, ncluster));
+        for (int b = 0; b < nbox; ++b)
+            if (cluster_idx[b] >= 0) B[b].cluster_active = ctx->coop_active + cluster_idx[b];
+        std::vector<int> one(ncluster, 1);
+        PM_CUDA(cudaMemcpy(ctx->coop_active, one.data(), sizeof(int) * ncluster, cudaMemcpyHostToDevice));
+    }
     // first iteration eagerly on the boxes' own streams (the autotuner runs here)
     for (int b = 0; b < nbox; ++b) {
         if (!B[b].active) continue;
-        Exec x(ctx, B[b].w->stream, B[b].w->partials, B[b].w->out, B[b].w->host, false);
+        Exec x = box_exec(ctx, B[b]);
         box_iteration(&x, B[b]);
     }
     for (int b = 0; b < nbox; ++b)
@@ -308,7 +328,7 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
     if (P.batch_persistent && !P.coarse_exact && P.coarsest_n == 4 && P.inner_cycles == 1) {
         std::vector<CoopBox> tab;
         for (int b = 0; b < nbox; ++b) {
-            if (!B[b].active || nn[b] < 2 * kCoopTop) continue;
+            if (!B[b].active || B[b].cluster || nn[b] < 2 * kCoopTop) continue;
             Workspace* w = B[b].w;
             const int l32 = coop_level(nn[b]);
             if ((int)w->s.size() != l32 + kCoopLevels) continue;
@@ -358,7 +378,7 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
             cudaStreamCaptureStatus cs;
             cudaStreamGetCaptureInfo(ms, &cs, nullptr, &cg, nullptr, nullptr, nullptr);
             std::set<cudaGraphNode_t> seen;
-            auto new_nodes = [&](std::vector<cudaGraphNode_t>& out) {
+            auto new_nodes = [&](std::vector<cudaGraphNode_t>& out, auto&& keep) {
                 size_t nn = 0;
                 cudaGraphGetNodes(cg, nullptr, &nn);
                 std::vector<cudaGraphNode_t> all(nn);
@@ -367,12 +387,20 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                     if (!seen.insert(nd).second) continue;
                     cudaGraphNodeType ty;
                     cudaGraphNodeGetType(nd, &ty);
-                    if (ty == cudaGraphNodeTypeKernel || ty == cudaGraphNodeTypeMemset || ty == cudaGraphNodeTypeMemcpy)
+                    if (ty == cudaGraphNodeTypeKernel ? keep(nd)
+                                                      : (ty == cudaGraphNodeTypeMemset || ty == cudaGraphNodeTypeMemcpy))
                         out.push_back(nd);
                 }
             };
+            // a cluster launch cannot be disabled in the executable graph: it stays and reads its box's flag
+            auto is_cluster = [&](cudaGraphNode_t nd) {
+                cudaKernelNodeAttrValue v{};
+                return cudaGraphKernelNodeGetAttribute(nd, cudaLaunchAttributeClusterDimension, &v) == cudaSuccess &&
+                       v.clusterDim.x > 1;
+            };
             std::vector<cudaGraphNode_t> dummy;
-            new_nodes(dummy);  // the fork
+            auto not_cluster = [&](cudaGraphNode_t nd) { return !is_cluster(nd); };
+            new_nodes(dummy, not_cluster);  // the fork
             std::vector<cudaEvent_t> joins;
             auto join_into_ms = [&](cudaStream_t st) {
                 cudaEvent_t join;
@@ -393,11 +421,11 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                 Workspace* w = B[b].w;
                 const pm_profile pb = ctx->prof;
                 cudaStreamWaitEvent(w->stream, fork, 0);
-                Exec x(ctx, w->stream, w->partials, w->out, w->host, false);
+                Exec x = box_exec(ctx, B[b]);
                 if (coop_idx[b] >= 0) box_down(&x, B[b], coop_level(nn[b]));
                 else box_iteration(&x, B[b]);
                 join_into_ms(w->stream);
-                new_nodes(box_nodes[b]);
+                new_nodes(box_nodes[b], not_cluster);
                 add_prof(b, pb);
                 enabled[b] = 1;
             }
@@ -441,7 +469,7 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                 cudaMemcpyAsync(ctx->coop_err_host, ctx->coop_bar + 2, sizeof(int), cudaMemcpyDeviceToHost, ms);
                 {
                     std::vector<cudaGraphNode_t> shared;  // the memset, kernel and copy belong to no box
-                    new_nodes(shared);
+                    new_nodes(shared, not_cluster);
                 }
                 cudaEvent_t fork2;
                 cudaEventCreateWithFlags(&fork2, cudaEventDisableTiming);
@@ -453,10 +481,10 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                     Workspace* w = B[b].w;
                     const pm_profile pb = ctx->prof;
                     cudaStreamWaitEvent(w->stream, fork2, 0);
-                    Exec x(ctx, w->stream, w->partials, w->out, w->host, false);
+                    Exec x = box_exec(ctx, B[b]);
                     box_up(&x, B[b], coop_level(nn[b]), cur32);
                     join_into_ms(w->stream);
-                    new_nodes(box_nodes[b]);
+                    new_nodes(box_nodes[b], not_cluster);
                     add_prof(b, pb);
                 }
             }
@@ -486,10 +514,12 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                 for (auto nd : box_nodes[b]) PM_CUDA(cudaGraphNodeSetEnabled(exec, nd, 0));
                 enabled[b] = 0;
             }
-        if (ncoop > 0) {
-            for (int b = 0; b < nbox; ++b)
-                if (coop_idx[b] >= 0) ctx->coop_active_host[coop_idx[b]] = B[b].active ? 1 : 0;
-            PM_CUDA(cudaMemcpyAsync(ctx->coop_active, ctx->coop_active_host, sizeof(int) * ncoop,
+        if (ncoop + ncluster > 0) {
+            for (int b = 0; b < nbox; ++b) {
+                const int k = coop_idx[b] >= 0 ? coop_idx[b] : cluster_idx[b];
+                if (k >= 0) ctx->coop_active_host[k] = B[b].active ? 1 : 0;
+            }
+            PM_CUDA(cudaMemcpyAsync(ctx->coop_active, ctx->coop_active_host, sizeof(int) * (ncoop + ncluster),
                                     cudaMemcpyHostToDevice, ctx->batch_stream));
         }
         PM_CUDA(cudaGraphLaunch(exec, ctx->batch_stream));
@@ -522,7 +552,7 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
     for (int b = 0; b < nbox; ++b) {
         if (B[b].trivial || !B[b].w) continue;
         BoxRun& R = B[b];
-        Exec x(ctx, R.w->stream, R.w->partials, R.w->out, R.w->host, false);
+        Exec x = box_exec(ctx, R);
         for (;;) {
             box_confirm(&x, R);
             PM_CUDA(cudaStreamSynchronize(R.w->stream));
@@ -538,6 +568,7 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                 R.st = PM_ERR_NOCONV;
                 break;
             }
+            x.cluster_active = nullptr;  // its flag may be down
             R.active = true;
             box_iteration(&x, R);
             PM_CUDA(cudaStreamSynchronize(R.w->stream));

@@ -228,6 +228,7 @@ struct pm_ctx {
     int coop_cap = 0;
     int coop_fail_block = -1, coop_fail_barrier = -1;
     double coop_wait_s = 2.0;
+    int cluster_ok = -1;  // whether the cluster of the coarse levels fits the device (-1: not asked yet)
     int conv_path = 0;  // convolution kernels of the U-Net call in progress (its pm_unet::conv_path)
     std::map<int, int> tuned;  // autotuned tile variant per (level size, inputs)
     std::string tune_log;
@@ -298,6 +299,8 @@ struct Exec {
     double* red_out;
     double* host_out;
     bool trace_ok;
+    bool cluster = false;  // the coarse inner levels run in one cluster launch (coarse_cluster.cuh)
+    const int* cluster_active = nullptr;  // its device flag (batched solves: 0 once the box has converged)
     const pm_params& prm;
     int num_sms;
     std::map<int, int>& tuned;

@@ -553,7 +553,7 @@ struct CoarsestSmem {
 
 // The coarsest solve of one level (at most 8^3 cells) by the calling block, its arrays in sm.
 template <typename T, bool BG>
-__device__ void coarsest_block(T* u, const T* F, T fscale, const uint8_t* kmask,
+__device__ __forceinline__ void coarsest_block(T* u, const T* F, T fscale, const uint8_t* kmask,
                                const T* bg, int n, double ih2_d, double nu_d, double kap_d, double eta,
                                int sweeps, bool floor_piece, CoarsestSmem<T>& sm, const K64& k64)
 {
@@ -610,51 +610,65 @@ __device__ void coarsest_block(T* u, const T* F, T fscale, const uint8_t* kmask,
             lsat[q] = kc[q] != T(0) ? (kmask ? lsat_c / w : lsat_c) : T(0);
         }
     }
-    auto stencil = [&](int q) {  // load_stencil's sums
-        const T* p = su + c[q];
-        const int xp = o[q][0], xm = o[q][1], yp = o[q][2], ym = o[q][3], zp = o[q][4], zm = o[q][5];
-        Stencil<T> s;
-        s.c0 = p[0];
-        s.ax = p[xp] + p[xm];
-        s.ay = p[yp] + p[ym];
-        s.az = p[zp] + p[zm];
-        s.exy = p[xp + yp] - p[xp + ym] - p[xm + yp] + p[xm + ym];
-        s.exz = p[xp + zp] - p[xp + zm] - p[xm + zp] + p[xm + zm];
-        s.eyz = p[yp + zp] - p[yp + zm] - p[ym + zp] + p[ym + zm];
-        return s;
-    };
     T lam = T(0);
+#pragma unroll 1
     for (int it = 0; it < sweeps && t < nt; ++it) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const Stencil<T> s = stencil(q);
-            T v;
-            if constexpr (sizeof(T) == 8)
-                v = s.c0 + update64(eval64(s, k64.nu1, k64.ep0, w64[q], f[q] + lam), k64, w64[q]);
-            else
-                v = s.c0 + local_update(local_eval<T, BG>(s, b[q], ih2, nu, kc[q], f[q] + lam, lsat[q]), sp, Df, ih2);
-            sync();
-            if (mine) su[c[q]] = v;
-            sync();
+        // steps 0, 1: the red and the black half-sweep; steps 2, 3: the pair's residuals.  One body for
+        // all four, because a single warp runs as fast as its instructions are fetched.
+        T a0 = T(0), a1 = T(0);
+#pragma unroll 1
+        for (int step = 0; step < 4; ++step) {
+            const bool q = step & 1;
+            const int cq = q ? c[1] : c[0];
+            const T* p = su + cq;
+            const int xp = q ? o[1][0] : o[0][0], xm = q ? o[1][1] : o[0][1], yp = q ? o[1][2] : o[0][2],
+                      ym = q ? o[1][3] : o[0][3], zp = q ? o[1][4] : o[0][4], zm = q ? o[1][5] : o[0][5];
+            Stencil<T> s;  // load_stencil's sums
+            s.c0 = p[0];
+            s.ax = p[xp] + p[xm];
+            s.ay = p[yp] + p[ym];
+            s.az = p[zp] + p[zm];
+            s.exy = p[xp + yp] - p[xp + ym] - p[xm + yp] + p[xm + ym];
+            s.exz = p[xp + zp] - p[xp + zm] - p[xm + zp] + p[xm + zm];
+            s.eyz = p[yp + zp] - p[yp + zm] - p[ym + zp] + p[ym + zm];
+            const T rhs = (q ? f[1] : f[0]) + lam;
+            T v = T(0), rv = T(0);
+            bool fl = false;
+            if constexpr (sizeof(T) == 8) {
+                const KW64 w{q ? w64[1].m2 : w64[0].m2, q ? w64[1].p8 : w64[0].p8, q ? w64[1].p96 : w64[0].p96,
+                             q ? w64[1].lsat : w64[0].lsat};
+                const Eval64 e = eval64(s, k64.nu1, k64.ep0, w, rhs);
+                if (step < 2) v = s.c0 + update64(e, k64, w);
+                else rv = resid64(e, k64, w, floor_piece ? k64.Df : 0.0, fl);
+            } else {
+                Stencil<T> g;
+                if (BG) {
+                    g.c0 = q ? b[1].c0 : b[0].c0;
+                    g.ax = q ? b[1].ax : b[0].ax;
+                    g.ay = q ? b[1].ay : b[0].ay;
+                    g.az = q ? b[1].az : b[0].az;
+                    g.exy = q ? b[1].exy : b[0].exy;
+                    g.exz = q ? b[1].exz : b[0].exz;
+                    g.eyz = q ? b[1].eyz : b[0].eyz;
+                }
+                const Local<T> e = local_eval<T, BG>(s, g, ih2, nu, q ? kc[1] : kc[0], rhs, q ? lsat[1] : lsat[0]);
+                if (step < 2) {
+                    v = s.c0 + local_update(e, sp, Df, ih2);
+                } else {
+                    fl = (e.P != T(0)) && (e.D < (floor_piece ? Df : T(0)));
+                    rv = fl ? nu * e.g : -e.G;
+                }
+            }
+            if (step < 2) {
+                sync();
+                if (mine) su[cq] = v;
+                sync();
+            } else {
+                a0 += mine ? rv : T(0);
+                a1 += mine && !fl ? T(1) : T(0);
+            }
         }
         // gauge update from the residual
-        T a0 = T(0), a1 = T(0);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const Stencil<T> s = stencil(q);
-            bool fl;
-            T rv;
-            if constexpr (sizeof(T) == 8) {
-                rv = resid64(eval64(s, k64.nu1, k64.ep0, w64[q], f[q] + lam), k64, w64[q],
-                             floor_piece ? k64.Df : 0.0, fl);
-            } else {
-                const Local<T> e = local_eval<T, BG>(s, b[q], ih2, nu, kc[q], f[q] + lam, lsat[q]);
-                fl = (e.P != T(0)) && (e.D < (floor_piece ? Df : T(0)));
-                rv = fl ? nu * e.g : -e.G;
-            }
-            a0 += mine ? rv : T(0);
-            a1 += mine && !fl ? T(1) : T(0);
-        }
         for (int d = 16; d > 0; d >>= 1) {
             a0 += __shfl_xor_sync(0xffffffffu, a0, d);
             a1 += __shfl_xor_sync(0xffffffffu, a1, d);
@@ -1024,6 +1038,12 @@ __global__ void k_add_correction_centred(double* __restrict__ x, const float* __
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x)
         x[c] += (double)e[c] - mean;
 }
+
+}  // namespace pmeft
+
+#include "coarse_cluster.cuh"
+
+namespace pmeft {
 
 // ------------------------------------------------------------------ host drivers
 
@@ -1638,10 +1658,71 @@ static void level_up(Exec* ctx, std::vector<Level<T>>& lv, int l, const T* F0, T
     for (int s = 0; s < ctx->prm.npost; ++s) sweep(ctx, L, F, fs, lam, c);
 }
 
+// Whether the hierarchy's levels from 32^3 down may run in the cluster launch: a coarse 32^3 level
+// with the default coarsest grid and its sweeps.  x->cluster is set by the solve that wants it.
+static bool cluster_levels(Exec* x, const std::vector<Level<float>>& s)
+{
+    if (x->prm.coarse_exact || x->prm.coarsest_n != 4 || s.empty() || s[0].n < 64 || !cluster_available(x->c))
+        return false;
+    for (const Level<float>& L : s)
+        if (L.n == 32) return L.u[0] && L.f && L.bg && L.kmask && !L.gap && !L.coef;
+    return false;
+}
+
+// The levels 32^3 .. 4^3 of the FP32 inner cycle in one launch, L the 32^3 level.
+static void coarse_cluster(Exec* ctx, Level<float>& L, const Coef& c)
+{
+    ClusterParams p{};
+    p.u = L.u[L.cur];
+    p.f = L.f;
+    p.bg = L.bg;
+    p.kmask = L.kmask;
+    p.active = ctx->cluster_active;
+    p.nu = (float)c.nu;
+    p.kap = (float)c.kap;
+    p.lsat_c = p.kap != 0.f ? (float)(0.75 * c.nu * (1.0 - c.eta) / c.kap) : 0.f;
+    p.nu_d = c.nu;
+    p.kap_d = c.kap;
+    p.eta = c.eta;
+    p.npre = ctx->prm.npre;
+    p.npost = ctx->prm.npost;
+    p.coarse_sweeps = ctx->prm.coarse_sweeps;
+    cudaLaunchConfig_t lc{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {kClBlocks, 1, 1};
+    lc.gridDim = dim3(kClBlocks);
+    lc.blockDim = dim3(kClThreads);
+    lc.dynamicSmemBytes = sizeof(ClSmem);
+    lc.stream = ctx->stream;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    ctx->begin(PM_K_SWEEP32, false, 0);
+    cudaLaunchKernelEx(&lc, k_coarse_cluster, p);  // a failure surfaces at the caller's next check
+    ctx->end();
+}
+
+// The background's restriction to the coarse inner levels (to 32^3 where the cluster launch forms
+// the ones below).
+static void restrict_background(Exec* x, std::vector<Level<float>>& s)
+{
+    for (size_t l = 0; l + 1 < s.size() && !(x->cluster && s[l].n <= 32); ++l) {
+        x->begin(PM_K_TRANSFER, false, 0);
+        k_restrict<float><<<grid_for(x, s[l + 1].cells), kThreads, 0, x->stream>>>(s[l].bg, s[l + 1].n, s[l + 1].bg);
+        x->end();
+    }
+}
+
 template <typename T>
 static void vcycle(Exec* ctx, std::vector<Level<T>>& lv, int l, const T* F0, T fs0, T lam0, const Coef& c)
 {
     Level<T>& L = lv[l];
+    if constexpr (sizeof(T) == 4) {
+        if (ctx->cluster && L.n == 32) {
+            coarse_cluster(ctx, L, c);
+            return;
+        }
+    }
     const T* F = l == 0 ? F0 : L.f;
     const T fs = l == 0 ? fs0 : T(1);
     const T lam = l == 0 ? lam0 : T(0);
@@ -1825,6 +1906,7 @@ pm_status mg_solve(pm_ctx* pctx, const double* delta, int n, const pm_coeffs& cf
     const bool mixed = P.precision >= 1;
     const bool ffo = P.precision == 1;
     PM_TRY(ensure_mg(pctx, w, mixed));
+    if (mixed) ex.cluster = cluster_levels(ctx, w->s);
     // The BF16 background coefficients of the finest inner level are written by the
     // float-float residual only: with the FP64 outer residual that level sweeps through the
     // background's own planes (the coefficient pointer is hidden for this solve).
@@ -1935,12 +2017,7 @@ pm_status mg_solve(pm_ctx* pctx, const double* delta, int n, const pm_coeffs& cf
         if (mixed) {
             // inner FP32 FAS V-cycle on the correction e, background chi32, rhs rplain - gm
             std::vector<Level<float>>& s = w->s;
-            for (size_t l = 0; l + 1 < s.size(); ++l) {
-                ctx->begin(PM_K_TRANSFER, false, 0);
-                k_restrict<float><<<grid_for(ctx, s[l + 1].cells), kThreads, 0, ctx->stream>>>(s[l].bg, s[l + 1].n,
-                                                                                               s[l + 1].bg);
-                ctx->end();
-            }
+            restrict_background(ctx, s);
             start_at_zero(ctx, s[0]);
             PM_CUDA(cudaGetLastError());
             for (int k = 0; k < P.inner_cycles; ++k) {
