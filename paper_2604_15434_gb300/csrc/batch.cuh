@@ -155,10 +155,7 @@ static void box_confirm(Exec* x, BoxRun& B)
 {
     Workspace* w = B.w;
     Level<double>& L0 = w->d[0];
-    x->begin(PM_K_REDUCE);
-    k_from_ff<<<grid_for(x, B.cells), kThreads, 0, x->stream>>>(ff_chi(w), B.cells, L0.u[0]);
-    x->end();
-    recentre<double>(x, L0.u[0], B.cells);
+    result_ff(x, ff_chi(w), B.cells, L0.u[0]);
     L0.lamp = w->lam;
     residual<double, false, false>(x, L0, L0.u[0], B.delta, B.cf.src, 0.0, B.c, nullptr, nullptr);
     L0.lamp = nullptr;
@@ -234,23 +231,19 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
         // kernel of all boxes, which holds every box up (24 boxes: 0.56 ms per iteration)
         Exec x = box_exec(ctx, R);
         R.cluster = x.cluster = P.batch_persistent && ctx->coop_fail_block < 0 && cluster_levels(&x, w->s);
-        PM_TRY(source_norm(&x, R.delta, R.cells, R.cf.src, &R.fnorm));
+        source_norm(&x, R.delta, R.cells);
         w->d[0].cur = 0;
         R.fk = make_ffcoef(R.cf.nu, R.cf.kappa, P.eta, nn[b]);
-        PM_CUDA(cudaMemcpyAsync(w->d[0].u[0], R.phi, R.cells * sizeof(double), cudaMemcpyDeviceToDevice, w->stream));
-        recentre<double>(&x, w->d[0].u[0], R.cells);
-        x.begin(PM_K_REDUCE);
-        k_to_ff<<<grid_for(&x, R.cells), kThreads, 0, w->stream>>>(R.delta, R.cf.src, R.cells, ff_rhs(w));
-        x.end();
-        x.begin(PM_K_REDUCE);
-        k_to_ff<<<grid_for(&x, R.cells), kThreads, 0, w->stream>>>(w->d[0].u[0], 1.0, R.cells, ff_chi(w));
-        x.end();
+        start_ff(&x, R.delta, R.cf.src, R.phi, R.cells, ff_rhs(w), ff_chi(w));
         PM_CUDA(cudaMemsetAsync(w->lam, 0, sizeof(double), w->stream));
         box_residual(&x, R);
         R.active = true;
     }
     for (int b = 0; b < nbox; ++b)
-        if (B[b].active) PM_CUDA(cudaStreamSynchronize(B[b].w->stream));
+        if (B[b].active) {
+            PM_CUDA(cudaStreamSynchronize(B[b].w->stream));
+            B[b].fnorm = source_norm_value(B[b].w->host, B[b].cf.src);
+        }
     // a guess worse than chi = 0 (or non-finite) is replaced by zero, as in the single solve
     bool redo = false;
     for (int b = 0; b < nbox; ++b) {
@@ -549,12 +542,17 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
     }
     // FP64 result of every box; a converged box's stop test is confirmed by its FP64
     // residual (a box that misses it by rounding gets further outer iterations, eagerly)
+    for (int b = 0; b < nbox; ++b) {  // side by side on the boxes' streams
+        if (B[b].trivial || !B[b].w) continue;
+        Exec x = box_exec(ctx, B[b]);
+        box_confirm(&x, B[b]);
+    }
     for (int b = 0; b < nbox; ++b) {
         if (B[b].trivial || !B[b].w) continue;
         BoxRun& R = B[b];
         Exec x = box_exec(ctx, R);
-        for (;;) {
-            box_confirm(&x, R);
+        for (bool again = false;; again = true) {
+            if (again) box_confirm(&x, R);
             PM_CUDA(cudaStreamSynchronize(R.w->stream));
             if (R.st != PM_OK) break;
             double gm64 = 0.0;
@@ -582,8 +580,9 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
     for (int b = 0; b < nbox; ++b) {
         if (B[b].trivial) continue;
         Workspace* w = B[b].w;
-        PM_CUDA(cudaMemcpyAsync(B[b].phi, w->d[0].u[0], B[b].cells * sizeof(double), cudaMemcpyDeviceToDevice,
-                                w->stream));
+        Exec x = box_exec(ctx, B[b]);
+        centre_into(&x, w->d[0].u[0], B[b].cells, B[b].phi);
+        PM_CUDA(cudaGetLastError());
         double lam = 0.0;
         PM_CUDA(cudaMemcpyAsync(&lam, w->lam, sizeof(double), cudaMemcpyDeviceToHost, w->stream));
         PM_CUDA(cudaStreamSynchronize(w->stream));

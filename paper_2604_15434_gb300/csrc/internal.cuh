@@ -36,6 +36,24 @@ constexpr int kMaxPartials = 4096;  // blocks of a reduction launch (fixed => de
 // floored cells is exactly 1) is replaced by chi = 0 before the first cycle.
 constexpr double kGuessLimit = 2.0;
 
+// ------------------------------------------------------------------ conversions
+//
+// A conversion between double and float or integer costs a slot of the FP64 pipe (16 cycles per warp
+// and SM); for ordinary values the integer pipe does it on the bits.
+
+// (double)f.  The conversion of the rare values is a call so that the compiler does not issue it for
+// the others as well.
+__device__ __noinline__ inline double f2d_rare(float f) { return (double)f; }
+__device__ __forceinline__ double f2d_bits(float f)
+{
+    const unsigned b = __float_as_uint(f), e = b & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) {  // zero; subnormal, infinite or not a number
+        if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+        return f2d_rare(f);
+    }
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+
 // ------------------------------------------------------------------ block reductions
 
 // 8 running sums per block: [0] sum r, [1] sum r over unfloored, [2] sum r^2,
@@ -69,14 +87,17 @@ __device__ __forceinline__ double rows_sum(const double* rows, int count, int q)
 // rows, the last group sums the groups' rows, both in a fixed order.
 //
 // FP64 additions bound this, not the data: the FP64 pipe takes 16 cycles per warp instruction
-// and SM.  So the threads' values go through shared memory and one warp sums each quantity (21
+// and SM.  So the threads' values go through shared memory and one warp sums each quantity (13
 // FP64 instructions per quantity and block of FP32 values; a shuffle tree in every warp took
 // 53), and the tail sums 2 x 64 rows by one warp per quantity instead of all rows in one block.
 // Measured against that form: mixed solve at 128^3 10.05 -> 8.70 ms; at 512^3 the 22 restricting
 // residuals 12.0 -> 11.0 ms, a sum of FP64 cells 0.53 -> 0.29 ms.
+// A single sum also leaves its mean over `count` values (fin_out[1], and as a float pair in the bits
+// of fin_out[2]): formed here once, where every thread of the kernels that use it would spend a
+// dozen FP64 instructions on the division.
 template <int NV, typename V>
 __device__ __forceinline__ void block_sums(const V (&v)[NV], double* partials, unsigned block,
-                                           double* fin_out = nullptr)
+                                           double* fin_out = nullptr, double count = 0.0)
 {
     __shared__ V sh[NV][256];
     __shared__ double tot[NV];
@@ -88,7 +109,10 @@ __device__ __forceinline__ void block_sums(const V (&v)[NV], double* partials, u
     for (int q = wid; q < NV; q += nw) {
         double s = 0.0;
 #pragma unroll 8
-        for (int i = lane; i < nt; i += 32) s += (double)sh[q][i];
+        for (int i = lane; i < nt; i += 32) {
+            if constexpr (sizeof(V) == 4) s += f2d_bits(sh[q][i]);
+            else s += sh[q][i];
+        }
         s = warp_sum(s);
         if (lane == 0) partials[(size_t)block * 8 + q] = s;
     }
@@ -129,14 +153,21 @@ __device__ __forceinline__ void block_sums(const V (&v)[NV], double* partials, u
     __syncthreads();
     if (t == 0) {
         if constexpr (NV >= 4) fin_out[8] = tot[3] > 0.0 ? tot[0] / tot[3] : 0.0;
+        if constexpr (NV == 1) {
+            const double mean = tot[0] / count;
+            const float hi = (float)mean;
+            fin_out[1] = mean;
+            *reinterpret_cast<float2*>(fin_out + 2) = make_float2(hi, (float)(mean - (double)hi));
+        }
         tickets[kSumGroups] = 0u;
     }
 }
 
 template <int NV, typename V>
-__device__ __forceinline__ void block_sums(const V (&v)[NV], double* partials, double* fin_out = nullptr)
+__device__ __forceinline__ void block_sums(const V (&v)[NV], double* partials, double* fin_out = nullptr,
+                                           double count = 0.0)
 {
-    block_sums<NV>(v, partials, blockIdx.x, fin_out);
+    block_sums<NV>(v, partials, blockIdx.x, fin_out, count);
 }
 
 // Screening weight of a cell from its mask byte k: the cell keeps (8 - k)/8 of kappa,

@@ -967,15 +967,15 @@ __global__ void __launch_bounds__(256) k_sum(const T* __restrict__ x, size_t tot
         for (int e = 0; e < W; ++e) a[0] += q.e[e];
     }
     const T v[1] = {(a[0] + a[1]) + (a[2] + a[3])};
-    block_sums<1>(v, partials, fin_out);
+    block_sums<1>(v, partials, fin_out, (double)total);
 }
 
-// sum of (x - mean)^2 with the mean read from the device
+// sum of (x - mean)^2 with the mean read from the device (sums[1], as k_sum leaves it)
 __global__ void __launch_bounds__(256) k_sum_centred(const double* __restrict__ x, size_t total,
                                                      const double* __restrict__ sums, double* __restrict__ partials,
                                                      double* __restrict__ fin_out)
 {
-    const double mean = sums[0] / (double)total;
+    const double mean = sums[1];
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -994,13 +994,13 @@ __global__ void __launch_bounds__(256) k_sum_centred(const double* __restrict__ 
         a[0] += d * d;
     }
     const double v[1] = {(a[0] + a[1]) + (a[2] + a[3])};
-    block_sums<1>(v, partials, fin_out);
+    block_sums<1>(v, partials, fin_out, 1.0);
 }
 
 template <typename T>
 __global__ void k_sub_mean(T* __restrict__ x, size_t total, const double* __restrict__ sums)
 {
-    const T mean = (T)(sums[0] / (double)total);
+    const T mean = (T)sums[1];
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x)
         x[c] -= mean;
 }
@@ -1030,11 +1030,11 @@ __global__ void k_bg_coef(const float* __restrict__ bg, int n, uint32_t* __restr
     }
 }
 
-// x += e - <e> in FP64, the mean of e read from the device (sums[0] = sum e)
+// x += e - <e> in FP64, the mean of e read from the device (sums[1])
 __global__ void k_add_correction_centred(double* __restrict__ x, const float* __restrict__ e, size_t total,
                                          const double* __restrict__ sums)
 {
-    const double mean = sums[0] / (double)total;
+    const double mean = sums[1];
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x)
         x[c] += (double)e[c] - mean;
 }
@@ -1779,13 +1779,51 @@ static int sum_grid(Exec* ctx, size_t cells)
     return g < cap ? g : cap;
 }
 
+// blocks of a pass with four cells per thread
+static unsigned grid4(size_t cells) { return (unsigned)((cells + 1023) / 1024); }
+
+// sum of x into red_out[16]
+template <typename T>
+static void field_sum(Exec* ctx, const T* x, size_t cells)
+{
+    ctx->begin(PM_K_REDUCE, false, 0);
+    k_sum<T><<<sum_grid(ctx, cells), kThreads, 0, ctx->stream>>>(x, cells, ctx->red_partials, ctx->red_out + 16);
+    ctx->end();
+}
+
+// float-float right-hand side src delta and centred guess of a mixed solve
+static void start_ff(Exec* ctx, const double* delta, double src, const double* guess, size_t cells, float2* rhs,
+                     float2* chi)
+{
+    field_sum<double>(ctx, guess, cells);
+    ctx->begin(PM_K_REDUCE, false, 0);
+    k_to_ff<true><<<grid4(cells), kThreads, 0, ctx->stream>>>(guess, 1.0, ctx->red_out + 16, cells, chi);
+    ctx->end();
+    ctx->begin(PM_K_REDUCE, false, 0);
+    k_to_ff<false><<<grid4(cells), kThreads, 0, ctx->stream>>>(delta, src, nullptr, cells, rhs);
+    ctx->end();
+}
+
+// the FP64 value of the float-float iterate in x, its sum in red_out[40]
+static void result_ff(Exec* ctx, const float2* chi, size_t cells, double* x)
+{
+    ctx->begin(PM_K_REDUCE, false, 0);
+    k_from_ff<<<std::min(grid_for(ctx, cells), 8 * ctx->num_sms), kThreads, 0, ctx->stream>>>(chi, cells, x, ctx->red_partials, ctx->red_out + 40);
+    ctx->end();
+}
+
+// phi = x - <x> from the sum result_ff left: <chi> = 0 to FP64 rounding
+static void centre_into(Exec* ctx, const double* x, size_t cells, double* phi)
+{
+    ctx->begin(PM_K_REDUCE, false, 0);
+    k_centre<<<grid4(cells), kThreads, 0, ctx->stream>>>(x, cells, ctx->red_out + 40, phi);
+    ctx->end();
+}
+
 template <typename T>
 static void recentre(Exec* ctx, T* x, size_t cells)
 {
-    const int grid = sum_grid(ctx, cells);
-    ctx->begin(PM_K_REDUCE, false, 0);
-    k_sum<T><<<grid, kThreads, 0, ctx->stream>>>(x, cells, ctx->red_partials, ctx->red_out + 16);
-    ctx->end();
+    field_sum<T>(ctx, x, cells);
     ctx->begin(PM_K_REDUCE, false, 0);
     k_sub_mean<T><<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(x, cells, ctx->red_out + 16);
     ctx->end();
@@ -1798,8 +1836,8 @@ static pm_status read_sums(Exec* ctx, int count)
     return PM_OK;
 }
 
-// |f - <f>|_2 for f = src * delta
-static pm_status source_norm(Exec* ctx, const double* delta, size_t cells, double src, double* out)
+// |delta - <delta>|_2^2 into host_out[48], valid after the stream's next synchronisation
+static void source_norm(Exec* ctx, const double* delta, size_t cells)
 {
     const int grid = sum_grid(ctx, cells);
     ctx->begin(PM_K_REDUCE, false, 0);
@@ -1809,11 +1847,10 @@ static pm_status source_norm(Exec* ctx, const double* delta, size_t cells, doubl
     k_sum_centred<<<grid, kThreads, 0, ctx->stream>>>(delta, cells, ctx->red_out + 32, ctx->red_partials,
                                                        ctx->red_out + 48);
     ctx->end();
-    PM_CUDA(cudaMemcpyAsync(ctx->host_out, ctx->red_out + 48, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    PM_CUDA(cudaStreamSynchronize(ctx->stream));
-    *out = std::fabs(src) * std::sqrt(ctx->host_out[0]);
-    return PM_OK;
+    cudaMemcpyAsync(ctx->host_out + 48, ctx->red_out + 48, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
 }
+// |f - <f>|_2 for f = src delta
+static double source_norm_value(const double* host, double src) { return std::fabs(src) * std::sqrt(host[48]); }
 
 // float-float outer residual of the mixed path (outer_ff.cuh); sums into red_out[0..8].
 // With a pending correction e (n >= kFzTX only; <e> already summed into red_out[16]) the
@@ -1849,10 +1886,7 @@ static void residual_ff(Exec* ctx, Workspace* w, const float2* xff, const float2
 // sum of the correction e into red_out[16]
 static void correction_sum(Exec* ctx, const float* e, size_t cells)
 {
-    const int grid = sum_grid(ctx, cells);
-    ctx->begin(PM_K_REDUCE, false, 0);
-    k_sum<float><<<grid, kThreads, 0, ctx->stream>>>(e, cells, ctx->red_partials, ctx->red_out + 16);
-    ctx->end();
+    field_sum<float>(ctx, e, cells);
 }
 
 // chi += e - <e> on the float-float iterate
@@ -1860,7 +1894,7 @@ static void add_correction_ff(Exec* ctx, float2* xff, const float* e, size_t cel
 {
     correction_sum(ctx, e, cells);
     ctx->begin(PM_K_REDUCE, false, 0);
-    k_add_correction_ff<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(xff, e, cells, ctx->red_out + 16);
+    k_add_correction_ff<<<grid4(cells), kThreads, 0, ctx->stream>>>(xff, e, cells, ctx->red_out + 16);
     ctx->end();
 }
 
@@ -1929,23 +1963,16 @@ pm_status mg_solve(pm_ctx* pctx, const double* delta, int n, const pm_coeffs& cf
     cudaEventRecord(e0, ctx->stream);
     Coef c{cf.nu, cf.kappa, P.eta, cf.src};
     double fnorm = 0.0;
-    PM_TRY(source_norm(ctx, delta, cells, cf.src, &fnorm));
+    source_norm(ctx, delta, cells);
     Level<double>& L0 = w->d[0];
     L0.cur = 0;
-    PM_CUDA(cudaMemcpyAsync(L0.u[0], phi, cells * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
+    if (!ffo)
+        PM_CUDA(cudaMemcpyAsync(L0.u[0], phi, cells * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     float2* xff = ffo ? ff_chi(w) : nullptr;
     float2* fff = ffo ? ff_rhs(w) : nullptr;
     const FFCoef fk = make_ffcoef(cf.nu, cf.kappa, P.eta, n);
     if (mixed && !ffo) recentre<double>(ctx, L0.u[0], cells);
-    if (ffo) {
-        recentre<double>(ctx, L0.u[0], cells);
-        ctx->begin(PM_K_REDUCE, false, 0);
-        k_to_ff<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(delta, cf.src, cells, fff);
-        ctx->end();
-        ctx->begin(PM_K_REDUCE, false, 0);
-        k_to_ff<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(L0.u[0], 1.0, cells, xff);
-        ctx->end();
-    }
+    if (ffo) start_ff(ctx, delta, cf.src, phi, cells, fff, xff);
     double lam = 0.0, rr = 0.0;
     int cyc = 0, vcyc = 0;
     pm_status st = PM_ERR_NOCONV;
@@ -1967,6 +1994,7 @@ pm_status mg_solve(pm_ctx* pctx, const double* delta, int n, const pm_coeffs& cf
             residual<double, false, false>(ctx, L0, L0.u[L0.cur], delta, cf.src, lam, c, nullptr, nullptr);
         PM_TRY(read_sums(ctx, 9));
         const double* h = ctx->host_out;
+        fnorm = source_norm_value(h, cf.src);
         double gm = 0.0;
         rr = rel_from_sums(h, fnorm, &gm);
         lam -= gm;
@@ -1996,9 +2024,7 @@ pm_status mg_solve(pm_ctx* pctx, const double* delta, int n, const pm_coeffs& cf
                 break;
             }
             // confirm the float-float stop test with the FP64 residual of the FP64 result
-            ctx->begin(PM_K_REDUCE, false, 0);
-            k_from_ff<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(xff, cells, L0.u[0]);
-            ctx->end();
+            result_ff(ctx, xff, cells, L0.u[0]);
             residual<double, false, false>(ctx, L0, L0.u[0], delta, cf.src, lam, c, nullptr, nullptr);
             PM_TRY(read_sums(ctx, 9));
             double gm64 = 0.0;
@@ -2045,16 +2071,13 @@ pm_status mg_solve(pm_ctx* pctx, const double* delta, int n, const pm_coeffs& cf
         ++cyc;
     }
     if (ffo) {
-        if (st != PM_OK) {
-            ctx->begin(PM_K_REDUCE, false, 0);
-            k_from_ff<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(xff, cells, L0.u[0]);
-            ctx->end();
-        }
-        recentre<double>(ctx, L0.u[0], cells);  // <chi> = 0 to FP64 rounding
-    } else if (mixed) {
-        recentre<double>(ctx, L0.u[L0.cur], cells);
+        if (st != PM_OK) result_ff(ctx, xff, cells, L0.u[0]);
+        centre_into(ctx, L0.u[0], cells, phi);
+    } else {
+        if (mixed) recentre<double>(ctx, L0.u[L0.cur], cells);
+        PM_CUDA(cudaMemcpyAsync(phi, L0.u[L0.cur], cells * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     }
-    PM_CUDA(cudaMemcpyAsync(phi, L0.u[L0.cur], cells * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
+    PM_CUDA(cudaGetLastError());
     cudaEventRecord(e1, ctx->stream);
     PM_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;

@@ -108,21 +108,88 @@ inline FFCoef make_ffcoef(double nu, double kap, double eta, int n)
     return c;
 }
 
-// y = ff(scale * x)
-__global__ void k_to_ff(const double* __restrict__ x, double scale, size_t total, float2* __restrict__ y)
+// v as a float pair, hi the nearest float (ties away from zero) and lo the nearest float of the rest,
+// on the integer and FP32 pipes; values outside 2^+-70 by conversions.
+__device__ __noinline__ inline float2 ff_rare(double v)
 {
-    for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x) {
-        const ff v = ff_from_double(scale * x[c]);
-        y[c] = make_float2(v.hi, v.lo);
+    const ff r = ff_from_double(v);
+    return make_float2(r.hi, r.lo);
+}
+__device__ __forceinline__ float2 ff_bits(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7ff) - 1023;
+    if (e < -70 || e > 70) {
+        if ((b << 1) == 0ull) return make_float2(0.f, 0.f);
+        return ff_rare(v);
     }
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const unsigned h = (unsigned)((m + 0x10000000ull) >> 29);  // 24 bits, rounded; 2^24 carries into the exponent
+    const int r = (int)((long long)m - ((long long)h << 29));  // |r| <= 2^28
+    const float hi = __uint_as_float((((unsigned)(e + 126) << 23) + h) | sign);
+    const float lo = __fmul_rn((float)r, __uint_as_float(((unsigned)(e + 75) << 23) | sign));  // r 2^(e - 52)
+    return make_float2(hi, lo);
 }
 
-__global__ void k_from_ff(const float2* __restrict__ x, size_t total, double* __restrict__ y)
+// y = ff(scale x), or ff(x - <x>) with <x> in sums[1] (CENTRE; sums as k_sum leaves them).  One FP64 operation per value;
+// bound by HBM (512^3: 1.22 -> 0.30 ms with the split on the integer pipe; of a zero guess 0.52).
+template <bool CENTRE>
+__global__ void __launch_bounds__(256) k_to_ff(const double* __restrict__ x, double scale,
+                                               const double* __restrict__ sums, size_t total, float2* __restrict__ y)
 {
-    for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x) {
-        const float2 v = x[c];
-        y[c] = (double)v.x + (double)v.y;
+    const double mean = CENTRE ? sums[1] : 0.0;
+    const size_t c0 = (size_t)blockIdx.x * 1024 + threadIdx.x;  // total is a multiple of 512
+    double v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c0 + 256 * k < total) v[k] = x[c0 + 256 * k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c0 + 256 * k < total) y[c0 + 256 * k] = ff_bits(CENTRE ? v[k] - mean : scale * v[k]);
+}
+
+// y = the FP64 value of x, its sum into fin_out[0]
+__global__ void __launch_bounds__(256) k_from_ff(const float2* __restrict__ x, size_t total, double* __restrict__ y,
+                                                 double* __restrict__ partials, double* __restrict__ fin_out)
+{
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; c + 3 * stride < total; c += 4 * stride) {
+        float2 q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q[k] = x[c + k * stride];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double v = f2d_bits(q[k].x) + f2d_bits(q[k].y);
+            a[k] += v;
+            y[c + k * stride] = v;
+        }
     }
+    for (; c < total; c += stride) {
+        const float2 q = x[c];
+        const double v = f2d_bits(q.x) + f2d_bits(q.y);
+        a[0] += v;
+        y[c] = v;
+    }
+    const double v[1] = {(a[0] + a[1]) + (a[2] + a[3])};
+    block_sums<1>(v, partials, fin_out, (double)total);
+}
+
+// y = x - <x>, <x> in sums[1]
+__global__ void __launch_bounds__(256) k_centre(const double* __restrict__ x, size_t total,
+                                                const double* __restrict__ sums, double* __restrict__ y)
+{
+    const double mean = sums[1];
+    const size_t c0 = (size_t)blockIdx.x * 1024 + threadIdx.x;
+    double v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c0 + 256 * k < total) v[k] = x[c0 + 256 * k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c0 + 256 * k < total) y[c0 + 256 * k] = v[k] - mean;
 }
 
 // chi += e - <e>, the correction of one outer iteration; subtracting the correction's
@@ -130,16 +197,26 @@ __global__ void k_from_ff(const float2* __restrict__ x, size_t total, double* __
 __global__ void k_add_correction_ff(float2* __restrict__ x, const float* __restrict__ e, size_t total,
                                     const double* __restrict__ sums)
 {
-    const double mean = sums[0] / (double)total;
-    const float mhi = (float)mean, mlo = (float)(mean - (double)mhi);
-    for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x) {
-        const float2 v = x[c];
-        float err;
-        const float s = ff_two_sum(e[c], -mhi, err);
-        const ff d = ff_norm(s, __fsub_rn(err, mlo));
-        const ff r = ff_add(ff{v.x, v.y}, d);
-        x[c] = make_float2(r.hi, r.lo);
-    }
+    const float2 mean = *reinterpret_cast<const float2*>(sums + 2);
+    const float mhi = mean.x, mlo = mean.y;
+    const size_t c0 = (size_t)blockIdx.x * 1024 + threadIdx.x;  // four cells per thread in flight
+    float2 v[4];
+    float d[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c0 + 256 * k < total) {
+            v[k] = x[c0 + 256 * k];
+            d[k] = e[c0 + 256 * k];
+        }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c0 + 256 * k < total) {
+            float err;
+            const float s = ff_two_sum(d[k], -mhi, err);
+            const ff t = ff_norm(s, __fsub_rn(err, mlo));
+            const ff r = ff_add(ff{v[k].x, v[k].y}, t);
+            x[c0 + 256 * k] = make_float2(r.hi, r.lo);
+        }
 }
 
 // Outer residual of the defect correction in float-float, with the same outputs as the
@@ -358,9 +435,9 @@ __global__ void __launch_bounds__(256, 3) k_residual_ff_zm(const float2* __restr
     const unsigned se_s = (unsigned)__cvta_generic_to_shared(se);
     float mhi = 0.f, mlo = 0.f;  // <E> as a float-float pair
     if (CORR) {
-        const double mean = esum[0] / ((double)n * n * n);
-        mhi = (float)mean;
-        mlo = (float)(mean - (double)mhi);
+        const float2 mean = *reinterpret_cast<const float2*>(esum + 2);
+        mhi = mean.x;
+        mlo = mean.y;
     }
     const int m = n - 1;
     const int x0 = blockIdx.x * kFzTX, y0 = blockIdx.y * kFzTY, z0 = blockIdx.z * NZ;
