@@ -14,14 +14,16 @@
 //      copied per tap, and each input plane is loaded once per column (plus two halo planes
 //      per work item) instead of three times.
 //   B: the layer's weights for NT output channels, resident for the block's lifetime, as
-//      [tap][chunk][k-half][co] x 16 bytes (stride 128 bytes per 8 outputs).
-// Pipeline per plane z: the block waits (bounded) for plane z - 1's MMAs, starts the copy of
-// plane z + SLOTS - 2 into the slot plane z - 2 left (SLOTS - 3 planes are in flight), waits for
-// plane z + 1, then one thread issues the
-// 27 x chunks MMAs of plane z into one of two tensor-memory accumulators (128 lanes x NT FP32
-// columns each) and commits them to that accumulator's mbarrier, while every warp reads plane
-// z - 1's 32 rows from the other accumulator with tcgen05.ld, adds the bias, applies ReLU / the
-// mask and stores BF16.  So the tensor core, the copies and the epilogue overlap.
+//      [in-plane tap][chunk][k-half][z tap][co] x 16 bytes (stride 128 bytes per 8 outputs).
+// Roles: three warps copy input planes, one thread watches the barriers, one issues MMAs, two groups of
+// four warps read finished output planes back in turn; they meet only at mbarriers, so copies, tensor
+// core and epilogue run at their own pace.  What bounds it is shared memory: an MMA of N = 48 reads 4 KB
+// of A and 1.5 KB of B and takes 57 cycles, one of N = 96 78.  When the same warps did everything in
+// turn, plane by plane, the tensor pipe was 21 to 35% busy (now 27 to 43).  Moving the window of output
+// planes costs the tensor core some 500 cycles more per input plane, which a second block on the SM
+// fills where two fit (16 -> 16 channels at 256^3: one block 0.52 ms, two 0.36).
+// Before -> now: 256^3 16 -> 16 channels 0.41 -> 0.36 ms, 48 -> 16 1.36 -> 0.80; 128^3 96 -> 32 0.79 -> 0.54,
+// 32 -> 32 0.17 -> 0.12; the warm start of a 256^3 box with the passes fused below 5.2 -> 3.6 ms.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -33,8 +35,10 @@ namespace pmeft {
 constexpr int kUmTX = 8, kUmTY = 16;                       // output tile (x, y), one z plane
 constexpr int kUmPX = kUmTX + 2, kUmPY = kUmTY + 2;
 constexpr int kUmPP = kUmPX * kUmPY;                       // 180 voxels per patch plane
-constexpr int kUmThreads = 128;
-constexpr long long kUmSpin = 1ll << 26;                   // bound on an mbarrier wait (polls)
+constexpr int kUmEpi = 128, kUmLoad = 96;                  // threads of an epilogue group, copying threads
+constexpr int kUmThreads = 2 * kUmEpi + 64 + kUmLoad;      // warps 0-3 and 4-7 (epilogue), 8 (MMA issue), 9-11
+                                                           // (copies), 12 (lookout)
+constexpr long long kUmSpin = 1ll << 22;                   // bound on an mbarrier wait (polls)
 
 __device__ __forceinline__ uint32_t um_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -106,242 +110,349 @@ __device__ __forceinline__ void um_st16_zero(uint32_t taddr)
         : "memory");
 }
 
-// weights held per (in-plane tap, chunk, k-half): the NT-row blocks of the z taps in the order
-// dz = 2, 1, 0, 2, 1, so that every rotation of (2, 1, 0) is a window of three blocks
-constexpr int kUmWGroups = 5;
-
-// dynamic shared memory of k_conv3d_umma for Cin input channels, NT outputs and SLOTS patch
-// planes: the resident weights, the planes, one mbarrier, the tensor-memory address and the NT
-// biases
-template <int NT, int SLOTS>
-constexpr size_t umma_smem(int cin)
+__device__ __forceinline__ void um_arrive(uint64_t* mbar)
 {
-    return (size_t)9 * (cin / 16) * 2 * kUmWGroups * NT * 16 + (size_t)SLOTS * (cin / 16) * kUmPP * 32 + 32 + NT * 4;
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(um_smem(mbar)) : "memory");
 }
 
-// tensor-memory columns of the block: three output planes of NT FP32 columns each, the
-// allocation a power of two of at least 32
-template <int NT>
-constexpr uint32_t um_cols()
+// BPS blocks share an SM's 512 tensor-memory columns; the output planes of NT columns each that a block
+// holds, a power of two
+template <int NT, int BPS>
+constexpr int um_planes()
 {
-    return 3 * NT <= 32 ? 32 : (3 * NT <= 64 ? 64 : (3 * NT <= 128 ? 128 : 256));
+    return (NT <= 16 ? 32 : (NT <= 32 ? 16 : 8)) / BPS;
 }
+
+constexpr int kUmMaxSlots = 8;  // input planes in flight
+// barriers: full and done per input slot, accumulator full and empty per output plane
+constexpr int kUmBars = 2 * kUmMaxSlots + 2 * 32;
+
+// dynamic shared memory of k_conv3d_umma for Cin input channels, NT outputs and `slots` patch planes:
+// the resident weights, the planes, the barriers, the tensor-memory address, a failure flag, biases
+inline size_t umma_smem(int nt, int cin, int slots)
+{
+    return (size_t)9 * (cin / 16) * 2 * 3 * nt * 16 + (size_t)slots * (cin / 16) * kUmPP * 32 + kUmBars * 8 + 16 + nt * 4;
+}
+
+// shared memory for each of `blocks` blocks on an SM (1 KB per block is the system's)
+inline size_t umma_budget(int blocks) { return (size_t)(228 / blocks - 1) * 1024; }
+
+// Where a convolution's input comes from and what else its epilogue makes (forward passes that keep
+// no activations for a backward pass; null / 0 otherwise).
+struct UmmaFuse {
+    // the first up_chunks 16-channel chunks come from `up` on the grid of half the size (nearest
+    // upsampling: voxel v reads its parent), the rest from `in`; the upsampled tensor is never stored
+    const __nv_bfloat16* up = nullptr;
+    int up_ld = 0, up_chunks = 0;
+    // the input holds 8 channels per voxel; the chunk's other 8 are zero
+    bool half = false;
+    // T[v] = sum_c head[c] y[v][c] + head[16] of the rounded outputs y (NT = 16) instead of storing them
+    const float* head = nullptr;
+    double* T = nullptr;
+};
 
 // out[v][out_off + co0 + c] = act(sum_tap sum_ci in[v + tap][ci] W[tap][ci][co0 + c] + bias[co0 + c]),
 // c < NT (NT <= 64), optionally times (mask[v][mask_off + co0 + c] > 0); bias may be null (no bias
 // term).  wt: the packed weights [tap][Cin/16][Cout][16] of the whole layer (Cout outputs).
-// Work item: an 8 x 16 column of outputs over zl planes (zl divides n).
+// Work item: an 8 x 16 column of outputs over zl planes (zl divides n, at most um_planes<NT, BPS>()).
 //
-// The block walks the input planes p = zs - 1 .. zs + zl of its column.  Input plane p feeds
-// output planes p + 1, p, p - 1 through the z taps dz = 0, 1, 2, so for each in-plane tap
-// (dy, dx) and chunk one MMA of N = 3 NT (B = the three z taps' weight blocks side by side)
-// adds its A operand, read once from shared memory, into all three outputs.  Each output plane
-// z keeps NT tensor-memory columns at slot (z - zs) mod 3; the B window is chosen so that the
-// three column groups of an MMA land in the slots of the right planes, and every MMA
-// accumulates (a slot is zeroed when its plane starts).  Output plane p - 2 is complete after
-// input plane p - 1's MMAs: the block waits (bounded) for them, reads that slot back with
-// tcgen05.ld (bias, ReLU / mask, BF16 stores), zeroes it for plane p + 1, starts the copy of
-// input plane p + SLOTS - 1, waits for plane p, and one thread issues plane p's 9 x chunks
-// MMAs.  Several blocks per SM overlap one block's epilogue with another's MMAs.
-// err (nullable): set to 1 if an mbarrier wait gave up (the block then stops; what it has not
+// The block walks the input planes p = zs - 1 .. zs + zl of its column.  Input plane p feeds output
+// planes p - 1, p, p + 1 through the z taps 2, 1, 0, so for each in-plane tap (dy, dx) and chunk one MMA
+// of N = 3 NT (B = the three z taps' weight blocks side by side) adds its A operand, read once from
+// shared memory, into all three outputs.  Output plane z keeps NT tensor-memory columns at slot z - zs,
+// so the three are neighbours; at the ends of the column the window is cut to the planes that exist.
+// Every MMA accumulates: the epilogue zeroes a slot as it empties it.
+//
+//   copying warps   wait done(slot) of the slot's last plane, copy plane p, arrive full(slot)
+//   lookout         wait full(slot) and empty(p + 1) in order, publish the number of planes that are ready
+//   MMA thread      read that number (one plane ahead of its use), issue plane p's MMAs, commit
+//                   done(slot) and acc(p - 1), which plane p completes
+//   epilogue warps  wait acc(z), read slot z, zero it, arrive empty(z), store plane z (each group every
+//                   other plane)
+//
+// err (nullable): set to 1 if a wait gave up (bounded polls; every role then leaves, what is not
 // written stays unwritten).
-template <int NT, int SLOTS>
-__global__ void __launch_bounds__(kUmThreads) k_conv3d_umma(const __nv_bfloat16* __restrict__ in, int in_ld, int in_off,
-                                                            int Cin, const __nv_bfloat16* __restrict__ wt, int Cout,
-                                                            int co0, const float* __restrict__ bias,
-                                                            __nv_bfloat16* __restrict__ out, int out_ld, int out_off,
-                                                            int n, int zl, int relu,
-                                                            const __nv_bfloat16* __restrict__ mask, int mask_ld,
-                                                            int mask_off, int* __restrict__ err)
+template <int NT, int BPS, bool FUSE>
+__global__ void __launch_bounds__(kUmThreads, BPS)
+    k_conv3d_umma(const __nv_bfloat16* __restrict__ in, int in_ld, int in_off, int Cin,
+                  const __nv_bfloat16* __restrict__ wt, int Cout, int co0, const float* __restrict__ bias,
+                  __nv_bfloat16* __restrict__ out, int out_ld, int out_off, int n, int zl, int slots, int relu,
+                  const __nv_bfloat16* __restrict__ mask, int mask_ld, int mask_off, int* __restrict__ err,
+                  UmmaFuse fuse)
 {
     static_assert(NT % 16 == 0 && NT >= 16 && NT <= 64, "N = 3 NT of a kind::f16 MMA with M = 128");
-    static_assert(SLOTS >= 2, "the plane the MMAs read and at least one loading");
-    constexpr int P = SLOTS - 1;  // planes loaded ahead of the one the MMAs read
-    constexpr uint32_t kCols = um_cols<NT>();
+    constexpr uint32_t kUmCols = 512 / BPS;
     extern __shared__ __align__(128) unsigned char um_raw[];
     const int kch = Cin / 16;
     const uint32_t slot_bytes = (uint32_t)kch * 2 * kUmPP * 16;
-    const uint32_t slot16 = slot_bytes >> 4;  // one patch-plane slot in 16-byte units
-    unsigned char* sW = um_raw;                                               // [9][kch][2][5 NT] x 16 B
-    unsigned char* sP = sW + (size_t)9 * kch * 2 * kUmWGroups * NT * 16;      // [slot][kch][2][PY][PX] x 16 B
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(sP + (size_t)SLOTS * slot_bytes);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2);
-    float* sBias = reinterpret_cast<float*>(mbar + 4);  // [NT]
+    unsigned char* sW = um_raw;                                      // [9][kch][2][3 NT] x 16 B
+    unsigned char* sP = sW + (size_t)9 * kch * 2 * 3 * NT * 16;      // [slot][kch][2][PY][PX] x 16 B
+    uint64_t* full = reinterpret_cast<uint64_t*>(sP + (size_t)slots * slot_bytes);
+    uint64_t* done = full + kUmMaxSlots;
+    uint64_t* acc = done + kUmMaxSlots;   // [32]
+    uint64_t* empty = acc + 32;           // [32]
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(empty + 32);
+    volatile int* failed = reinterpret_cast<volatile int*>(tslot + 1);
+    uint32_t* ready = tslot + 2;  // input planes of this block ready for the tensor core so far
+    float* sBias = reinterpret_cast<float*>(tslot + 4);  // [NT]
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const uint32_t sW_s = um_smem(sW), sP_s = um_smem(sP);
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(um_smem(tslot)),
-                     "r"(kCols));
+                     "r"(kUmCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (t == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(um_smem(mbar)), "r"(1));
+        *failed = 0;
+        *ready = 0;
+        for (int q = 0; q < kUmMaxSlots; ++q) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(um_smem(full + q)), "r"(kUmLoad));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(um_smem(done + q)), "r"(1));
+        }
+        for (int q = 0; q < 32; ++q) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(um_smem(acc + q)), "r"(1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(um_smem(empty + q)), "r"(kUmEpi));
+        }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");  // visible to the tensor core's arrive
     }
     if (bias)
         for (int c = t; c < NT; c += kUmThreads) sBias[c] = bias[co0 + c];
-    // resident weights: 16-byte piece (tap9, chunk, half, group, c) = output co0 + c of the z tap
-    // dz = (2 - group) mod 3 at in-plane tap tap9 = dy * 3 + dx
-    const int wpieces = 9 * kch * 2 * kUmWGroups * NT;
+    // resident weights: 16-byte piece (tap9, chunk, half, group, c) = output co0 + c of the z tap 2 - group
+    // at in-plane tap tap9 = dy * 3 + dx
+    const int wpieces = 9 * kch * 2 * 3 * NT;
     for (int q = t; q < wpieces; q += kUmThreads) {
-        const int c = q % NT, r = q / NT;  // r = ((tap9 * kch + ch) * 2 + half) * 5 + group
-        const int g = r % kUmWGroups, r2 = r / kUmWGroups;
-        const int half = r2 & 1, tc = r2 >> 1;  // tc = tap9 * kch + ch
-        const int tap9 = tc / kch, ch = tc - tap9 * kch;
-        const int dz = (2 - g + 3) % 3;
-        const int tap27 = dz * 9 + tap9;
-        const __nv_bfloat16* src = wt + (((size_t)tap27 * kch + ch) * Cout + co0 + c) * 16 + half * 8;
-        um_cp16(sW_s + (uint32_t)q * 16u, src);
+        const int c = q % NT, r = q / NT;  // r = ((tap9 * kch + ch) * 2 + half) * 3 + group
+        const int g = r % 3, r2 = r / 3, half = r2 & 1, tc = r2 >> 1;
+        const int tap9 = tc / kch, ch = tc - tap9 * kch, tap27 = (2 - g) * 9 + tap9;
+        um_cp16(sW_s + (uint32_t)q * 16u, wt + (((size_t)tap27 * kch + ch) * Cout + co0 + c) * 16 + half * 8);
     }
-    asm volatile("cp.async.commit_group;\n" ::);
+    if (FUSE && fuse.half)  // the upper 8 channels of every slot, never written again
+        for (int q = t; q < slots * kUmPP; q += kUmThreads)
+            *reinterpret_cast<uint4*>(sP + (size_t)(q / kUmPP) * slot_bytes + (size_t)(kUmPP + q % kUmPP) * 16) =
+                make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // visible to the tensor core
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = *tslot;
-
-    const int m = n - 1;
-    const int tx = n / kUmTX, ty = n / kUmTY, nzs = n / zl;
-    const long long items = (long long)tx * ty * nzs;
-    constexpr uint32_t idesc = um_idesc(128, 3 * NT);
-    // descriptors of the first A and B core matrices; the others differ only in the start
-    // address field (addresses below 256 KB, so adding (offset >> 4) never carries out of it)
-    const uint64_t dA0 = um_desc(sP_s, kUmPP * 16, kUmPX * 16);
-    const uint64_t dB0 = um_desc(sW_s, kUmWGroups * NT * 16, 128);
-    const int ppieces = kch * 2 * kUmPP;
-    uint32_t phase = 0;     // parity of the mbarrier's next completion
-    bool inflight = false;  // MMAs committed but not yet waited for
-    bool failed = false;
-
-    // all threads poll (bounded) for the completion of the committed MMAs
-    auto wait_mma = [&]() -> bool {
-        bool done = false;
-        for (long long it = 0; it < kUmSpin && !done; ++it) done = um_try_wait(mbar, phase);
-        if (done) {
-            phase ^= 1u;
-            inflight = false;
-        }
-        return done;
-    };
-
-    for (long long item = blockIdx.x; item < items && !failed; item += gridDim.x) {
-        const int bx = (int)(item % tx), by = (int)((item / tx) % ty), bz = (int)(item / ((long long)tx * ty));
-        const int x0 = bx * kUmTX, y0 = by * kUmTY, zs = bz * zl;
-        // input plane z (periodic) into slot sl: 16-byte piece (chunk, half, y, x); one copy group
-        auto load_plane = [&](int z, int sl) {
-            const uint32_t base = sP_s + (uint32_t)sl * slot_bytes;
-            const size_t zo = (size_t)(z & m) * n;
-            for (int q = t; q < ppieces; q += kUmThreads) {
-                const int p = q % kUmPP, r = q / kUmPP;  // r = chunk * 2 + half
-                const int px = p % kUmPX, py = p / kUmPX;
-                const size_t v = (zo + ((y0 - 1 + py) & m)) * n + ((x0 - 1 + px) & m);
-                um_cp16(base + (uint32_t)q * 16u, in + v * in_ld + in_off + r * 8);
-            }
-            asm volatile("cp.async.commit_group;\n" ::);
-        };
-        // tensor-memory column of output plane z's slot, for this warp's lanes
-        auto slot_addr = [&](int z) {
-            return tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(((z - zs + 3) % 3) * NT);
-        };
-        // the outputs of plane z from its slot: row warp * 32 + lane is voxel (x0 + row % 8,
-        // y0 + row / 8)
-        auto epilogue = [&](int z) {
-            const int row = warp * 32 + lane;
-            const int xv = x0 + (row & 7), yv = y0 + (row >> 3);
-            const size_t v = ((size_t)z * n + yv) * n + xv;
-#pragma unroll
-            for (int c0 = 0; c0 < NT; c0 += 16) {
-                float d[16];
-                um_ld16(slot_addr(z) + (uint32_t)c0, d);
-                __align__(16) __nv_bfloat16 o[16];
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    float y = bias ? d[q] + sBias[c0 + q] : d[q];  // no bias in the backward-data convolution
-                    if (relu) y = fmaxf(y, 0.f);
-                    if (mask && !(__bfloat162float(mask[v * mask_ld + mask_off + co0 + c0 + q]) > 0.f)) y = 0.f;
-                    o[q] = __float2bfloat16(y);
-                }
-                uint4* dst = reinterpret_cast<uint4*>(out + v * out_ld + out_off + co0 + c0);
-                dst[0] = reinterpret_cast<const uint4*>(o)[0];
-                dst[1] = reinterpret_cast<const uint4*>(o)[1];
-            }
-        };
-        // input plane p sits in slot (p - zs + 1) % SLOTS; planes zs - 1 .. zs - 1 + P first
-        for (int k = 0; k < P; ++k) load_plane(zs - 1 + k, k);
-        for (int p = zs - 1; p <= zs + zl; ++p) {
-            const int pr = p - zs + 1;  // 0 .. zl + 1
-            bool ok = true;
-            if (pr >= 1) {
-                // input plane p - 1's MMAs done: output plane p - 2 is complete, and plane p - 1's
-                // slot is free
-                ok = wait_mma();
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                if (ok && p - 2 >= zs) epilogue(p - 2);
-            }
-            // output plane p + 1 starts in the slot plane p - 2 leaves
-#pragma unroll
-            for (int c0 = 0; c0 < NT; c0 += 16) um_st16_zero(slot_addr(p + 1) + (uint32_t)c0);
-            asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-            if (p + P <= zs + zl) load_plane(p + P, (pr + P) % SLOTS);
-            else asm volatile("cp.async.commit_group;\n" ::);
-            // plane p has landed (the P newest groups may still be in flight)
-            asm volatile("cp.async.wait_group %0;\n" ::"n"(P) : "memory");
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // visible to the tensor core
-            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-            ok = __syncthreads_and(ok) != 0;
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            if (!ok) {  // block-uniform
-                failed = true;
-                break;
-            }
-            // plane p: 9 in-plane taps x kch chunks, N = 3 NT into the slots of planes p + 1, p, p - 1
-            if (t == 0) {
-                const int q3 = (p - zs + 3) % 3;
-                const int j = (4 - q3) % 3;  // B window: column group k gets dz = (2 - j - k) mod 3
-                const uint64_t ab = dA0 + (uint64_t)((uint32_t)(pr % SLOTS) * slot16);
-                const uint64_t bb = dB0 + (uint64_t)(j * NT);
-                const uint64_t bstep = (uint64_t)(kch * 2 * kUmWGroups * NT);  // one in-plane tap of B, 16-byte units
-                for (int ch = 0; ch < kch; ++ch) {
-                    const uint64_t ac = ab + (uint64_t)(ch * 2 * kUmPP);
-                    const uint64_t bc = bb + (uint64_t)(ch * 2 * kUmWGroups * NT);
-#pragma unroll
-                    for (int tap9 = 0; tap9 < 9; ++tap9) {
-                        const int dy = tap9 / 3, dx = tap9 % 3;
-                        um_mma(tmem, ac + (uint64_t)(dy * kUmPX + dx), bc + (uint64_t)tap9 * bstep, idesc, 1u);
-                    }
-                }
-                um_commit(mbar);
-            }
-            inflight = true;
-            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        }
-        if (failed) break;
-        // the last output plane
-        bool ok = wait_mma();
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        ok = __syncthreads_and(ok) != 0;
-        if (!ok) {
-            failed = true;
-            break;
-        }
-        epilogue(zs + zl - 1);
-        // every thread is done with the slots before the next item
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-    if (failed && t == 0) {
-        if (err) atomicExch(err, 1);
-        // give the MMAs still in flight one more bounded wait before their memory is released
-        if (inflight)
-            for (long long it = 0; it < kUmSpin; ++it)
-                if (um_try_wait(mbar, phase)) break;
+    if (warp < 4) {  // every output slot starts at zero
+        for (int c = 0; c < um_planes<NT, BPS>() * NT; c += 16) um_st16_zero(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c);
+        asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
+
+    const int m = n - 1;
+    const int tx = n / kUmTX, ty = n / kUmTY, nzs = n / zl;
+    const long long items = (long long)tx * ty * nzs;
+    // a bounded wait for the completion of a barrier's phase; false once any role has given up
+    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+        for (long long it = 0; it < kUmSpin; ++it) {
+            if (um_try_wait(bar, parity)) return true;
+            if (*failed) return false;
+        }
+        *failed = 1;
+        return false;
+    };
+    int slot = 0;            // input slot of the next plane and the parity of its use
+    uint32_t round = 0;
+    uint32_t use = 0;        // parity of this item's use of the output slots
+    auto next_slot = [&]() {
+        if (++slot == slots) {
+            slot = 0;
+            round ^= 1u;
+        }
+    };
+
+    if (warp == 12) {
+        // ---- lookout: a barrier poll costs the MMA thread some 200 cycles beside the operand reads, so this
+        // thread polls and the MMA thread loads a counter whose value it needs one plane later
+        if (lane == 0) {
+            bool ok = true;
+            uint32_t count = 0;
+            for (long long item = blockIdx.x; item < items && ok; item += gridDim.x, use ^= 1u)
+                for (int r = -1; r <= zl && ok; ++r) {
+                    ok = wait(full + slot, round);
+                    if (ok && r + 1 < zl) ok = wait(empty + (r + 1), use ^ 1u);
+                    if (ok) asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(um_smem(ready)), "r"(++count) : "memory");
+                    next_slot();
+                }
+        }
+    } else if (warp >= 9) {
+        // ---- copies: this thread's voxels of a plane, 48 voxels x 2 halves per pass; up to `lag` planes are
+        // in flight behind the newest, then handed over in order
+        const int lt = t - (2 * kUmEpi + 32), half = lt & 1;
+        const int lag = slots >= 6 ? 4 : (slots >= 4 ? 2 : 1);  // less than slots: the tensor core keeps one
+        int flying = 0, oldest = 0;
+        auto hand_over = [&]() {
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            um_arrive(full + oldest);
+            if (++oldest == slots) oldest = 0;
+            --flying;
+        };
+        bool ok = true;
+        for (long long item = blockIdx.x; item < items && ok; item += gridDim.x) {
+            const int x0 = (int)(item % tx) * kUmTX, y0 = (int)((item / tx) % ty) * kUmTY,
+                      zs = (int)(item / ((long long)tx * ty)) * zl;
+            int off[4], offu[4];  // of the voxel in a plane, and of its parent in a coarse plane
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int v = (lt >> 1) + 48 * i, py = v / kUmPX, px = v - py * kUmPX;
+                const int y = (y0 - 1 + py) & m, x = (x0 - 1 + px) & m;
+                off[i] = v < kUmPP && !(FUSE && fuse.half && half) ? (y * n + x) * in_ld + in_off + half * 8 : -1;
+                if (FUSE) offu[i] = ((y >> 1) * (n >> 1) + (x >> 1)) * fuse.up_ld + half * 8;
+            }
+            for (int p = zs - 1; p <= zs + zl; ++p) {
+                ok = wait(done + slot, round ^ 1u);  // the tensor core is done with the slot's last plane
+                if (!ok) break;
+                const __nv_bfloat16* src = in + (size_t)(p & m) * n * n * in_ld;
+                const __nv_bfloat16* srcu = FUSE ? fuse.up + (size_t)((p & m) >> 1) * (n >> 1) * (n >> 1) * fuse.up_ld : nullptr;
+                const int upc = FUSE ? fuse.up_chunks : 0;
+                const uint32_t dst = sP_s + (uint32_t)slot * slot_bytes + (uint32_t)(half * kUmPP + (lt >> 1)) * 16u;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (off[i] < 0) continue;
+                    for (int ch = 0; ch < upc; ++ch)
+                        um_cp16(dst + (uint32_t)(ch * 2 * kUmPP + 48 * i) * 16u, srcu + offu[i] + ch * 16);
+                    for (int ch = upc; ch < kch; ++ch)
+                        um_cp16(dst + (uint32_t)(ch * 2 * kUmPP + 48 * i) * 16u,
+                                src + off[i] + (ch - upc) * 16);
+                }
+                asm volatile("cp.async.commit_group;\n" ::);
+                ++flying;
+                if (flying > lag) {
+                    if (lag == 4) asm volatile("cp.async.wait_group 4;\n" ::: "memory");
+                    else if (lag == 2) asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+                    else asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                    hand_over();
+                }
+                next_slot();
+            }
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        while (flying > 0) hand_over();
+    } else if (warp == 8) {
+        if (lane == 0) {
+            // ---- MMA issue
+            // descriptors of the first A and B core matrices; the others differ only in the start
+            // address field (addresses below 256 KB, so adding (offset >> 4) never carries out of it)
+            const uint64_t dA0 = um_desc(sP_s, kUmPP * 16, kUmPX * 16);
+            const uint64_t dB0 = um_desc(sW_s, 3 * NT * 16, 128);
+            bool ok = true;
+            int last = -1;  // input slot and parity of the last plane issued
+            uint32_t last_round = 0;
+            uint32_t have = 0, mine = 0;  // planes known to be ready, planes issued
+            auto load_ready = [&]() {
+                uint32_t v;
+                asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(um_smem(ready)) : "memory");
+                return v;
+            };
+            for (long long item = blockIdx.x; item < items && ok; item += gridDim.x) {
+                for (int r = -1; r <= zl; ++r) {  // input plane zs + r, outputs r - 1 .. r + 1 of this column
+                    for (long long it = 0; have <= mine && ok; ++it) {
+                        have = load_ready();
+                        ok = it < kUmSpin && !*failed;
+                    }
+                    if (!ok) {
+                        *failed = 1;
+                        break;
+                    }
+                    ++mine;
+                    const uint32_t ahead = load_ready();  // used at the next plane
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const int z0 = max(r - 1, 0), z1 = min(r + 1, zl - 1);
+                    const uint32_t idesc = um_idesc(128, (z1 - z0 + 1) * NT), d = tmem + (uint32_t)(z0 * NT);
+                    const uint64_t ab = dA0 + (uint64_t)((uint32_t)slot * (slot_bytes >> 4));
+                    const uint64_t bb = dB0 + (uint64_t)((z0 - (r - 1)) * NT);
+                    const uint64_t bstep = (uint64_t)(kch * 2 * 3 * NT);  // one in-plane tap of B, 16-byte units
+                    for (int ch = 0; ch < kch; ++ch) {
+                        const uint64_t ac = ab + (uint64_t)(ch * 2 * kUmPP);
+                        const uint64_t bc = bb + (uint64_t)(ch * 2 * 3 * NT);
+#pragma unroll
+                        for (int tap9 = 0; tap9 < 9; ++tap9) {
+                            const int dy = tap9 / 3, dx = tap9 % 3;
+                            um_mma(d, ac + (uint64_t)(dy * kUmPX + dx), bc + (uint64_t)tap9 * bstep, idesc, 1u);
+                        }
+                    }
+                    um_commit(done + slot);
+                    if (r >= 1) um_commit(acc + (r - 1));
+                    last = slot;
+                    last_round = round;
+                    next_slot();
+                    have = ahead;
+                }
+            }
+            // the MMAs in flight end before the tensor memory is released (bounded, also after a failure)
+            if (last >= 0)
+                for (long long it = 0; it < kUmSpin; ++it)
+                    if (um_try_wait(done + last, last_round)) break;
+        }
+    } else {
+        // ---- epilogue: row warp * 32 + lane of an output plane is voxel (x0 + row % 8, y0 + row / 8)
+        const int row = t & (kUmEpi - 1), group = warp >> 2;
+        float hw[FUSE ? 17 : 1];
+        if (FUSE && fuse.T)
+#pragma unroll
+            for (int q = 0; q < 17; ++q) hw[FUSE ? q : 0] = fuse.head[q];
+        bool ok = true;
+        for (long long item = blockIdx.x; item < items && ok; item += gridDim.x, use ^= 1u) {
+            const int x0 = (int)(item % tx) * kUmTX, y0 = (int)((item / tx) % ty) * kUmTY,
+                      zs = (int)(item / ((long long)tx * ty)) * zl;
+            const size_t v0 = ((size_t)zs * n + y0 + (row >> 3)) * n + x0 + (row & 7);
+            for (int z = group; z < zl; z += 2) {
+                ok = wait(acc + z, use);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t ts = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(z * NT);
+                float d[NT];
+#pragma unroll
+                for (int c0 = 0; c0 < NT; c0 += 16) {
+                    float d16[16];
+                    um_ld16(ts + (uint32_t)c0, d16);
+                    um_st16_zero(ts + (uint32_t)c0);
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) d[c0 + q] = d16[q];
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                um_arrive(empty + z);
+                const size_t v = v0 + (size_t)z * n * n;
+#pragma unroll
+                for (int c0 = 0; c0 < NT; c0 += 16) {
+                    __align__(16) __nv_bfloat16 o[16];
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) {
+                        float y = bias ? d[c0 + q] + sBias[c0 + q] : d[c0 + q];  // no bias in the backward-data convolution
+                        if (relu) y = fmaxf(y, 0.f);
+                        if (mask && !(__bfloat162float(mask[v * mask_ld + mask_off + co0 + c0 + q]) > 0.f)) y = 0.f;
+                        o[q] = __float2bfloat16(y);
+                    }
+                    if (FUSE && fuse.T) {  // the head's sum, in its own kernel's order
+                        float h = hw[FUSE ? 16 : 0];
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) h += hw[FUSE ? q : 0] * __bfloat162float(o[q]);
+                        fuse.T[v] = (double)h;
+                        continue;
+                    }
+                    uint4* dst = reinterpret_cast<uint4*>(out + v * out_ld + out_off + co0 + c0);
+                    dst[0] = reinterpret_cast<const uint4*>(o)[0];
+                    dst[1] = reinterpret_cast<const uint4*>(o)[1];
+                }
+            }
+        }
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (t == 0 && *failed && err) atomicExch(err, 1);
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kUmCols));
 }
 
 }  // namespace pmeft

@@ -44,16 +44,16 @@ static long long total_params()
 // ---------------------------------------------------------------- small kernels
 
 __global__ void k_pack_input(const double* __restrict__ delta, int nvox, float p1, float p2, float p3,
-                             __nv_bfloat16* __restrict__ out)
+                             int ld, __nv_bfloat16* __restrict__ out)
 {
     // the network sees asinh(delta) in BF16: FP32 asinh is far below that rounding
     const __nv_bfloat16 b1 = __float2bfloat16(p1), b2 = __float2bfloat16(p2), b3 = __float2bfloat16(p3);
     const __nv_bfloat16 z = __float2bfloat16(0.f);
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += gridDim.x * blockDim.x) {
         __align__(16) __nv_bfloat16 o[8] = {__float2bfloat16(asinhf((float)delta[v])), b1, b2, b3, z, z, z, z};
-        uint4* dst = reinterpret_cast<uint4*>(out + (size_t)v * 16);
+        uint4* dst = reinterpret_cast<uint4*>(out + (size_t)v * ld);  // ld 8, or 16 with the rest zero
         dst[0] = *reinterpret_cast<const uint4*>(o);
-        dst[1] = make_uint4(0u, 0u, 0u, 0u);
+        if (ld == 16) dst[1] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -252,7 +252,8 @@ __global__ void k_target(const double* __restrict__ chi, int n, double scale, fl
 
 struct Acts {
     int n = 0;
-    __nv_bfloat16 *in = nullptr, *y0 = nullptr, *cat1 = nullptr, *p1 = nullptr, *y2 = nullptr, *cat2 = nullptr,
+    // skip1, skip2: c1's and c3's outputs alone, where the concatenations cat1, cat2 are not stored
+    __nv_bfloat16 *in = nullptr, *y0 = nullptr, *skip1 = nullptr, *skip2 = nullptr, *cat1 = nullptr, *p1 = nullptr, *y2 = nullptr, *cat2 = nullptr,
                   *p2 = nullptr, *y4 = nullptr, *y5 = nullptr, *y6 = nullptr, *y7 = nullptr, *y8 = nullptr,
                   *y9 = nullptr;
     // gradients (training)
@@ -290,7 +291,7 @@ static pm_status dalloc(pm_ctx* ctx, T** p, size_t count)
 
 static void free_acts(Acts& a)
 {
-    __nv_bfloat16** bufs[] = {&a.in, &a.y0, &a.cat1, &a.p1, &a.y2, &a.cat2, &a.p2, &a.y4, &a.y5, &a.y6, &a.y7, &a.y8,
+    __nv_bfloat16** bufs[] = {&a.in, &a.y0, &a.skip1, &a.skip2, &a.cat1, &a.p1, &a.y2, &a.cat2, &a.p2, &a.y4, &a.y5, &a.y6, &a.y7, &a.y8,
                               &a.y9, &a.d9, &a.d8, &a.dcat1, &a.d7, &a.d6, &a.dcat2, &a.d5, &a.d4, &a.dp2, &a.d2,
                               &a.dp1, &a.d0};
     for (auto b : bufs) {
@@ -306,29 +307,40 @@ static void free_acts(Acts& a)
 // the weight gradient's partial sums (chunks) for an n^3 level
 static int wgrad_rows(int n) { return (int)(((size_t)n * n * n + kWgChunk - 1) / kWgChunk); }
 
+// Whether level l (0 or 1) of a forward pass that keeps no activations reads its skip connection and the
+// coarser level directly (UmmaFuse) instead of a stored concatenation: where its convolutions take the
+// tcgen05 kernel.
+static bool unet_fused(const pm_unet* u, int n, int l, bool train)
+{
+    return !train && u->conv_path == 1 && (n >> l) >= kUmTY;
+}
+
 static pm_status ensure_acts(pm_unet* u, int n, bool train)
 {
     pm_ctx* ctx = u->ctx;
     Acts& a = u->acts;
-    if (a.n == n && (a.train || !train)) return PM_OK;
-    free_acts(a);
+    const bool f0 = unet_fused(u, n, 0, train), f1 = unet_fused(u, n, 1, train);
+    if (a.n == n && (a.train || !train) && (f0 ? a.skip1 : a.cat1) && (f1 ? a.skip2 : a.cat2) && (f0 || a.y9)) return PM_OK;
+    if (a.n != n || (train && !a.train)) free_acts(a);
+    train = train || a.train;  // a training set that lacks only the forward pass's buffers is kept
     const size_t v0 = (size_t)n * n * n, v1 = v0 / 8, v2 = v0 / 64;
-    PM_TRY(dalloc(ctx, &a.in, v0 * 16));
-    PM_TRY(dalloc(ctx, &a.y0, v0 * 16));
-    PM_TRY(dalloc(ctx, &a.cat1, v0 * 48));
-    PM_TRY(dalloc(ctx, &a.p1, v1 * 16));
-    PM_TRY(dalloc(ctx, &a.y2, v1 * 32));
-    PM_TRY(dalloc(ctx, &a.cat2, v1 * 96));
-    PM_TRY(dalloc(ctx, &a.p2, v2 * 32));
-    PM_TRY(dalloc(ctx, &a.y4, v2 * 64));
-    PM_TRY(dalloc(ctx, &a.y5, v2 * 64));
-    PM_TRY(dalloc(ctx, &a.y6, v1 * 32));
-    PM_TRY(dalloc(ctx, &a.y7, v1 * 32));
-    PM_TRY(dalloc(ctx, &a.y8, v0 * 16));
-    PM_TRY(dalloc(ctx, &a.y9, v0 * 16));
-    PM_TRY(dalloc(ctx, &a.that, v0));
-    PM_TRY(dalloc(ctx, &a.lpart, (size_t)kMaxPartials * 19));
-    if (train) {
+    auto want = [&](auto** p, size_t count) { return *p ? PM_OK : dalloc(ctx, p, count); };
+    PM_TRY(want(&a.in, v0 * 16));
+    PM_TRY(want(&a.y0, v0 * 16));
+    PM_TRY(f0 ? want(&a.skip1, v0 * 16) : want(&a.cat1, v0 * 48));
+    PM_TRY(want(&a.p1, v1 * 16));
+    PM_TRY(want(&a.y2, v1 * 32));
+    PM_TRY(f1 ? want(&a.skip2, v1 * 32) : want(&a.cat2, v1 * 96));
+    PM_TRY(want(&a.p2, v2 * 32));
+    PM_TRY(want(&a.y4, v2 * 64));
+    PM_TRY(want(&a.y5, v2 * 64));
+    PM_TRY(want(&a.y6, v1 * 32));
+    PM_TRY(want(&a.y7, v1 * 32));
+    PM_TRY(want(&a.y8, v0 * 16));
+    if (!f0) PM_TRY(want(&a.y9, v0 * 16));
+    PM_TRY(want(&a.that, v0));
+    PM_TRY(want(&a.lpart, (size_t)kMaxPartials * 19));
+    if (train && !a.train) {
         PM_TRY(dalloc(ctx, &a.d9, v0 * 16));
         PM_TRY(dalloc(ctx, &a.d8, v0 * 16));
         PM_TRY(dalloc(ctx, &a.dcat1, v0 * 48));
@@ -358,70 +370,61 @@ static pm_status ensure_acts(pm_unet* u, int n, bool train)
 
 static int blocks_for(pm_ctx* ctx, size_t work) { return grid_for(ctx, work); }
 
-// The convolution on the tcgen05 tensor cores (conv_umma.cuh), in slices of NT output channels
-// whose resident weights fit next to the patch planes in shared memory.  Returns false (nothing
-// launched) where it does not apply.
-template <int NT, int SLOTS>
+// The convolution on the tcgen05 tensor cores (conv_umma.cuh) for NT output channels from co0 on, BPS
+// blocks per SM.
+template <int NT, int BPS, bool FUSE = false>
 static void launch_umma(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off, int ci, const __nv_bfloat16* w,
                         int co, int co0, const float* bias, __nv_bfloat16* out, int out_ld, int out_off, int n, bool relu,
-                        const __nv_bfloat16* mask, int mask_ld, int mask_off)
+                        const __nv_bfloat16* mask, int mask_ld, int mask_off, const UmmaFuse& fuse)
 {
-    const size_t smem = umma_smem<NT, SLOTS>(ci);
-    auto k = k_conv3d_umma<NT, SLOTS>;
+    // as many patch planes as fit beside the weights; enough shared memory that no further block, for
+    // which there would be no tensor memory, sits on the SM
+    const size_t most = umma_budget(BPS);
+    int slots = kUmMaxSlots;
+    while (slots > 2 && umma_smem(NT, ci, slots) > most) --slots;
+    const size_t smem = std::max(umma_smem(NT, ci, slots), umma_budget(BPS + 1) + 1024);
+    auto k = k_conv3d_umma<NT, BPS, FUSE>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    // blocks per SM from the kernel's own limits: shared memory (plus the 1 KB the system
-    // reserves per block), registers, threads, and the SM's 512 tensor-memory columns
-    int smem_sm = 0, regs_sm = 0;
-    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
-    cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, ctx->device);
-    cudaFuncAttributes fa{};
-    cudaFuncGetAttributes(&fa, k);
-    constexpr int cols = (int)um_cols<NT>();
-    int per_sm = std::min(smem_sm / (int)(smem + 1024), 2048 / kUmThreads);
-    if (fa.numRegs > 0) per_sm = std::min(per_sm, regs_sm / (fa.numRegs * kUmThreads));
-    per_sm = std::max(1, std::min(per_sm, 512 / cols));
-    // z planes per work item: n / 8 within [4, 64] (a divisor of n), enough items for every SM
-    const int zl = std::max(4, std::min(64, n / 8));
+    // z planes per work item: the divisor of n, at most the tensor memory's output planes, with the
+    // fewest input planes (zl + 2 per item) on the busiest block
+    const long long blocks = (long long)ctx->num_sms * BPS;
+    int zl = 4;
+    long long best = 1ll << 60;
+    for (int c = 4; c <= um_planes<NT, BPS>() && c <= n; c *= 2) {
+        const long long items = (long long)(n / kUmTX) * (n / kUmTY) * (n / c);
+        const long long cost = (items + blocks - 1) / blocks * (c + 2);
+        if (cost <= best) {
+            best = cost;
+            zl = c;
+        }
+    }
     const long long items = (long long)(n / kUmTX) * (n / kUmTY) * (n / zl);
-    const long long g = std::min<long long>(items, (long long)ctx->num_sms * per_sm);
-    k<<<(int)g, kUmThreads, smem, ctx->stream>>>(in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, zl,
-                                                  relu ? 1 : 0, mask, mask_ld, mask_off, ctx->flag + 2);
+    k<<<(int)std::min<long long>(items, blocks), kUmThreads, smem, ctx->stream>>>(
+        in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, zl, slots, relu ? 1 : 0, mask, mask_ld,
+        mask_off, ctx->flag + 2, fuse);
 }
 
-// three plane slots (two planes loading ahead) where the block still fits twice per SM, else two
-template <int NT>
-static void launch_umma_slots(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off, int ci,
-                              const __nv_bfloat16* w, int co, int co0, const float* bias, __nv_bfloat16* out,
-                              int out_ld, int out_off, int n, bool relu, const __nv_bfloat16* mask, int mask_ld,
-                              int mask_off)
-{
-    if (umma_smem<NT, 3>(ci) <= (size_t)112 * 1024)
-        launch_umma<NT, 3>(ctx, in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, relu, mask, mask_ld,
-                           mask_off);
-    else
-        launch_umma<NT, 2>(ctx, in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, relu, mask, mask_ld,
-                           mask_off);
-}
-
+// In slices of NT output channels whose resident weights fit beside two patch planes.  Returns false
+// (nothing launched) where it does not apply.
 static bool conv_umma(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off, int ci, const __nv_bfloat16* w,
                       int co, const float* bias, __nv_bfloat16* out, int out_ld, int out_off, int n, bool relu,
-                      const __nv_bfloat16* mask, int mask_ld, int mask_off)
+                      const __nv_bfloat16* mask, int mask_ld, int mask_off, const UmmaFuse& fuse)
 {
     if (ctx->conv_path != 1 || n < kUmTY || n % kUmTY != 0 || ci % 16 != 0 || co % 16 != 0) return false;
-    auto bytes = [&](int nt) {  // umma_smem<nt, 2>(ci)
-        return (size_t)9 * (ci / 16) * 2 * kUmWGroups * nt * 16 + (size_t)2 * (ci / 16) * kUmPP * 32 + 32 + (size_t)nt * 4;
-    };
     int nt = co;  // the widest slice (at most 64 outputs) whose weights fit
-    while ((nt > 64 || bytes(nt) > (size_t)227 * 1024) && nt % 32 == 0) nt /= 2;
-    if (nt > 64 || bytes(nt) > (size_t)227 * 1024) return false;
+    while ((nt > 64 || umma_smem(nt, ci, 2) > (size_t)227 * 1024) && nt % 32 == 0) nt /= 2;
+    if (nt > 64 || umma_smem(nt, ci, 2) > (size_t)227 * 1024) return false;
     for (int co0 = 0; co0 < co; co0 += nt) {
-        switch (nt) {
-            case 16: launch_umma_slots<16>(ctx, in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off); break;
-            case 32: launch_umma_slots<32>(ctx, in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off); break;
-            case 48: launch_umma_slots<48>(ctx, in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off); break;
-            case 64: launch_umma_slots<64>(ctx, in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off); break;
-            default: return false;
-        }
+        const bool two = umma_smem(nt, ci, 4) <= umma_budget(2);
+        const bool fused = fuse.half || fuse.up || fuse.T;
+        if (fused && nt != 16) return false;
+        const auto launch = fused      ? (two ? launch_umma<16, 2, true> : launch_umma<16, 1, true>)
+                            : nt == 16   ? (two ? launch_umma<16, 2> : launch_umma<16, 1>)
+                            : nt == 32 ? (two ? launch_umma<32, 2> : launch_umma<32, 1>)
+                            : nt == 48 ? (two ? launch_umma<48, 2> : launch_umma<48, 1>)
+                                       : launch_umma<64, 1>;
+        launch(ctx, in, in_ld, in_off, ci, w, co, co0, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off,
+               fuse);
     }
     return true;
 }
@@ -429,11 +432,13 @@ static bool conv_umma(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_of
 // forward conv launcher (also the backward-data conv with a mask)
 static void conv_fwd(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off, int ci, const __nv_bfloat16* w,
                      int co, const float* bias, __nv_bfloat16* out, int out_ld, int out_off, int n, bool relu,
-                     const __nv_bfloat16* mask = nullptr, int mask_ld = 0, int mask_off = 0)
+                     const __nv_bfloat16* mask = nullptr, int mask_ld = 0, int mask_off = 0,
+                     const UmmaFuse& fuse = {})
 {
     const int nvox = n * n * n, grid = (nvox + kConvM - 1) / kConvM;
     ctx->begin(PM_K_PM);
-    if (conv_umma(ctx, in, in_ld, in_off, ci, w, co, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off)) {
+    if (conv_umma(ctx, in, in_ld, in_off, ci, w, co, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off,
+                  fuse)) {
         ctx->end();
         return;
     }
@@ -560,41 +565,60 @@ static pm_status umma_status(pm_ctx* ctx)
     return PM_OK;
 }
 
-static pm_status unet_forward(pm_unet* u, const double* delta, int n, double aB0, double aM0, double a)
+static pm_status unet_forward(pm_unet* u, const double* delta, int n, double aB0, double aM0, double a, bool train)
 {
     pm_ctx* ctx = u->ctx;
     ctx->conv_path = u->conv_path;  // the convolution launcher reads it from the context
     Acts& A = u->acts;
     const int n1 = n / 2, n2 = n / 4;
     const size_t v0 = (size_t)n * n * n;
+    // f0, f1: levels 0 and 1 without stored concatenations (256^3: upsampling 0.28 ms, pooling from a slice
+    // 0.25 -> 0.10, the padded input and the head 0.25 -> 0.08)
+    const bool f0 = unet_fused(u, n, 0, train), f1 = unet_fused(u, n, 1, train);
+    UmmaFuse half, up0, up1, head;
+    half.half = f0;
+    if (f0) up0.up = A.y7, up0.up_ld = 32, up0.up_chunks = 2;
+    if (f1) up1.up = A.y5, up1.up_ld = 64, up1.up_chunks = 4;
+    if (f0) head.head = u->p + u->off[10], head.T = A.that;
+    // the skip connections: alone, or in their slice of the concatenation
+    __nv_bfloat16 *s1 = f0 ? A.skip1 : A.cat1, *s2 = f1 ? A.skip2 : A.cat2;
+    const int s1_ld = f0 ? 16 : 48, s1_off = f0 ? 0 : 32, s2_ld = f1 ? 32 : 96, s2_off = f1 ? 0 : 64;
+    const int in_ld = f0 ? 8 : 16;
     ctx->begin(PM_K_PM);
-    k_pack_input<<<blocks_for(ctx, v0), 256, 0, ctx->stream>>>(delta, (int)v0, (float)aB0, (float)aM0, (float)a, A.in);
+    k_pack_input<<<blocks_for(ctx, v0), 256, 0, ctx->stream>>>(delta, (int)v0, (float)aB0, (float)aM0, (float)a, in_ld,
+                                                               A.in);
     ctx->end();
-    conv_fwd(ctx, A.in, 16, 0, 16, u->wf[0], 16, bias_of(u, 0), A.y0, 16, 0, n, true);
-    conv_fwd(ctx, A.y0, 16, 0, 16, u->wf[1], 16, bias_of(u, 1), A.cat1, 48, 32, n, true);
+    conv_fwd(ctx, A.in, in_ld, 0, 16, u->wf[0], 16, bias_of(u, 0), A.y0, 16, 0, n, true, nullptr, 0, 0, half);
+    conv_fwd(ctx, A.y0, 16, 0, 16, u->wf[1], 16, bias_of(u, 1), s1, s1_ld, s1_off, n, true);
     ctx->begin(PM_K_PM);
-    k_pool2<<<blocks_for(ctx, v0 / 8 * 16), 256, 0, ctx->stream>>>(A.cat1, 48, 32, 16, n, A.p1);
+    k_pool2<<<blocks_for(ctx, v0 / 8 * 16), 256, 0, ctx->stream>>>(s1, s1_ld, s1_off, 16, n, A.p1);
     ctx->end();
     conv_fwd(ctx, A.p1, 16, 0, 16, u->wf[2], 32, bias_of(u, 2), A.y2, 32, 0, n1, true);
-    conv_fwd(ctx, A.y2, 32, 0, 32, u->wf[3], 32, bias_of(u, 3), A.cat2, 96, 64, n1, true);
+    conv_fwd(ctx, A.y2, 32, 0, 32, u->wf[3], 32, bias_of(u, 3), s2, s2_ld, s2_off, n1, true);
     ctx->begin(PM_K_PM);
-    k_pool2<<<blocks_for(ctx, v0 / 64 * 32), 256, 0, ctx->stream>>>(A.cat2, 96, 64, 32, n1, A.p2);
+    k_pool2<<<blocks_for(ctx, v0 / 64 * 32), 256, 0, ctx->stream>>>(s2, s2_ld, s2_off, 32, n1, A.p2);
     ctx->end();
     conv_fwd(ctx, A.p2, 32, 0, 32, u->wf[4], 64, bias_of(u, 4), A.y4, 64, 0, n2, true);
     conv_fwd(ctx, A.y4, 64, 0, 64, u->wf[5], 64, bias_of(u, 5), A.y5, 64, 0, n2, true);
-    ctx->begin(PM_K_PM);
-    k_up2<<<blocks_for(ctx, v0 / 8 * 64), 256, 0, ctx->stream>>>(A.y5, 64, n2, A.cat2, 96, 0);
-    ctx->end();
-    conv_fwd(ctx, A.cat2, 96, 0, 96, u->wf[6], 32, bias_of(u, 6), A.y6, 32, 0, n1, true);
+    if (!f1) {
+        ctx->begin(PM_K_PM);
+        k_up2<<<blocks_for(ctx, v0 / 8 * 64), 256, 0, ctx->stream>>>(A.y5, 64, n2, A.cat2, 96, 0);
+        ctx->end();
+    }
+    conv_fwd(ctx, s2, s2_ld, 0, 96, u->wf[6], 32, bias_of(u, 6), A.y6, 32, 0, n1, true, nullptr, 0, 0, up1);
     conv_fwd(ctx, A.y6, 32, 0, 32, u->wf[7], 32, bias_of(u, 7), A.y7, 32, 0, n1, true);
-    ctx->begin(PM_K_PM);
-    k_up2<<<blocks_for(ctx, v0 * 32), 256, 0, ctx->stream>>>(A.y7, 32, n1, A.cat1, 48, 0);
-    ctx->end();
-    conv_fwd(ctx, A.cat1, 48, 0, 48, u->wf[8], 16, bias_of(u, 8), A.y8, 16, 0, n, true);
-    conv_fwd(ctx, A.y8, 16, 0, 16, u->wf[9], 16, bias_of(u, 9), A.y9, 16, 0, n, true);
-    ctx->begin(PM_K_PM);
-    k_head<<<blocks_for(ctx, v0), 256, 0, ctx->stream>>>(A.y9, u->p + u->off[10], (int)v0, A.that);
-    ctx->end();
+    if (!f0) {
+        ctx->begin(PM_K_PM);
+        k_up2<<<blocks_for(ctx, v0 * 32), 256, 0, ctx->stream>>>(A.y7, 32, n1, A.cat1, 48, 0);
+        ctx->end();
+    }
+    conv_fwd(ctx, s1, s1_ld, 0, 48, u->wf[8], 16, bias_of(u, 8), A.y8, 16, 0, n, true, nullptr, 0, 0, up0);
+    conv_fwd(ctx, A.y8, 16, 0, 16, u->wf[9], 16, bias_of(u, 9), A.y9, 16, 0, n, true, nullptr, 0, 0, head);
+    if (!f0) {
+        ctx->begin(PM_K_PM);
+        k_head<<<blocks_for(ctx, v0), 256, 0, ctx->stream>>>(A.y9, u->p + u->off[10], (int)v0, A.that);
+        ctx->end();
+    }
     PM_CUDA(cudaGetLastError());
     return umma_status(ctx);
 }
@@ -778,7 +802,7 @@ extern "C" pm_status pm_unet_forward(pm_unet* u, const double* delta, int n, dou
     if (!u || !delta || !T_out || !unet_n_ok(n)) return PM_ERR_INVALID_ARG;
     pm_ctx* ctx = u->ctx;
     PM_TRY(ensure_acts(u, n, false));
-    PM_TRY(unet_forward(u, delta, n, aB0, aM0, a));
+    PM_TRY(unet_forward(u, delta, n, aB0, aM0, a, false));
     PM_CUDA(cudaMemcpyAsync(T_out, u->acts.that, (size_t)n * n * n * sizeof(double), cudaMemcpyDeviceToDevice,
                             ctx->stream));
     return PM_OK;
@@ -789,7 +813,7 @@ extern "C" pm_status pm_unet_loss_grad(pm_unet* u, const double* delta, const fl
 {
     if (!u || !delta || !target || !loss || !unet_n_ok(n)) return PM_ERR_INVALID_ARG;
     PM_TRY(ensure_acts(u, n, true));
-    PM_TRY(unet_forward(u, delta, n, aB0, aM0, a));
+    PM_TRY(unet_forward(u, delta, n, aB0, aM0, a, true));
     return unet_backward(u, target, n, loss);
 }
 
@@ -841,7 +865,7 @@ extern "C" pm_status pm_unet_warm_start(pm_unet* u, const double* delta, int n, 
         return PM_OK;
     }
     PM_TRY(ensure_acts(u, n, false));
-    PM_TRY(unet_forward(u, delta, n, aB0, aM0, a));
+    PM_TRY(unet_forward(u, delta, n, aB0, aM0, a, false));
     // L chi_0 = (src / nu) T_hat, zero mean
     return poisson32(ctx, u->acts.that, n, cf.src / cf.nu, phi_out);
 }
