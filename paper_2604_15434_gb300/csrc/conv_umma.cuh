@@ -426,11 +426,17 @@ __global__ void __launch_bounds__(kUmThreads, BPS)
 #pragma unroll
                 for (int c0 = 0; c0 < NT; c0 += 16) {
                     __align__(16) __nv_bfloat16 o[16];
+                    __align__(16) __nv_bfloat16 mk[16];
+                    if (mask) {
+                        const uint4* src = reinterpret_cast<const uint4*>(mask + v * mask_ld + mask_off + co0 + c0);
+                        reinterpret_cast<uint4*>(mk)[0] = src[0];
+                        reinterpret_cast<uint4*>(mk)[1] = src[1];
+                    }
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
                         float y = bias ? d[c0 + q] + sBias[c0 + q] : d[c0 + q];  // no bias in the backward-data convolution
                         if (relu) y = fmaxf(y, 0.f);
-                        if (mask && !(__bfloat162float(mask[v * mask_ld + mask_off + co0 + c0 + q]) > 0.f)) y = 0.f;
+                        if (mask && !(__bfloat162float(mk[q]) > 0.f)) y = 0.f;
                         o[q] = __float2bfloat16(y);
                     }
                     if (FUSE && fuse.T) {  // the head's sum, in its own kernel's order
