@@ -199,7 +199,8 @@ __global__ void __launch_bounds__(256) k_residual64(const double* __restrict__ u
 // planes of its 32 x 8 tile and their one-cell halo in a shared ring, so each iterate value is
 // read from global memory once per block instead of once per stencil point.  Grid (n/32, n/8,
 // n/nz).  0.275 -> 0.156 ms at 128^3 with the arithmetic above (63 -> 33 FP64 instructions per
-// cell), 14.8 -> 8.6 ms for the confirming residual of a 512^3 mixed solve.  MIXED (precision 2) also writes the FP32 copies of the defect-correction loop.
+// cell), 14.8 -> 8.6 ms for the confirming residual of a 512^3 mixed solve.  MIXED (precision 2)
+// also writes the FP32 copies of the defect-correction loop.
 constexpr int kR64TX = 32, kR64TY = 8;
 template <bool WRITE_R, bool MIXED, bool MASK>
 __global__ void __launch_bounds__(256) k_residual64_zm(const double* __restrict__ u, const double* __restrict__ F,

@@ -7,7 +7,7 @@
 // shared memory in the K-major, unswizzled layout of the tensor core's descriptors: 8 rows of
 // 16 bytes (8 BF16 k-values) form a 128-byte core matrix; the leading byte offset steps to the
 // next 8 k, the stride byte offset to the next 8 rows.
-//   A: a block marches an 8 x 16 column of tiles up z.  It keeps SLOTS patch planes (10 x 18
+//   A: a block marches an 8 x 16 column of tiles up z.  It keeps up to eight patch planes (10 x 18
 //      voxels, periodic) in a ring, each as [chunk][k-half][y][x] x 16 bytes: eight consecutive
 //      x of one patch row are a core matrix, the next y row is the next one (stride 160 bytes),
 //      so the A operand of a tap is the plane z + dz with its start moved by (dy, dx); no data is
@@ -23,7 +23,8 @@
 // planes costs the tensor core some 500 cycles more per input plane, which a second block on the SM
 // fills where two fit (16 -> 16 channels at 256^3: one block 0.52 ms, two 0.36).
 // Before -> now: 256^3 16 -> 16 channels 0.41 -> 0.36 ms, 48 -> 16 1.36 -> 0.80; 128^3 96 -> 32 0.79 -> 0.54,
-// 32 -> 32 0.17 -> 0.12; the warm start of a 256^3 box with the passes fused below 5.2 -> 3.6 ms.
+// 32 -> 32 0.17 -> 0.12; the warm start of a 256^3 box with the passes fused below 5.2 -> 3.6 ms.  The epilogue
+// reads a data gradient's ReLU mask as two 16-byte loads: 16 -> 48 channels at 128^3 0.195 -> 0.118 ms.
 #pragma once
 
 #include <cuda_bf16.h>
