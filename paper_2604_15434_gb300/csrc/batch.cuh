@@ -58,7 +58,8 @@ static pm_status box_prepare(pm_ctx* ctx, Workspace* w)
     if (!w->stream) PM_CUDA(cudaStreamCreateWithFlags(&w->stream, cudaStreamNonBlocking));
     if (!w->partials) {
         PM_CUDA(cudaMalloc(&w->partials, sizeof(double) * kPartialsDoubles));
-        PM_CUDA(cudaMemset(w->partials, 0, sizeof(double) * kPartialsDoubles));  // with the launch counter
+        // with the launch counter; on the box's own stream, which nothing on the legacy stream is ordered before
+        PM_CUDA(cudaMemsetAsync(w->partials, 0, sizeof(double) * kPartialsDoubles, w->stream));
     }
     if (!w->out) PM_CUDA(cudaMalloc(&w->out, sizeof(double) * 64));
     if (!w->host) PM_CUDA(cudaMallocHost(&w->host, sizeof(double) * 64));
@@ -268,20 +269,8 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                 PM_CUDA(cudaStreamSynchronize(B[b].w->stream));
                 box_check(P, B[b], tol);
             }
-    // flags of the boxes whose coarse levels are cluster launches (these and the cooperative boxes share
-    // one array: either form serves all boxes of a call)
-    std::vector<int> cluster_idx(nbox, -1);
-    int ncluster = 0;
-    for (int b = 0; b < nbox; ++b)
-        if (B[b].active && B[b].cluster) cluster_idx[b] = ncluster++;
-    if (ncluster > 0) {
-        PM_TRY(coop_alloc(ctx, ncluster));
-        for (int b = 0; b < nbox; ++b)
-            if (cluster_idx[b] >= 0) B[b].cluster_active = ctx->coop_active + cluster_idx[b];
-        std::vector<int> one(ncluster, 1);
-        PM_CUDA(cudaMemcpy(ctx->coop_active, one.data(), sizeof(int) * ncluster, cudaMemcpyHostToDevice));
-    }
-    // first iteration eagerly on the boxes' own streams (the autotuner runs here)
+    // first iteration eagerly on the boxes' own streams (the autotuner runs here); every box in it is
+    // active, so its cluster launch reads no flag
     for (int b = 0; b < nbox; ++b) {
         if (!B[b].active) continue;
         Exec x = box_exec(ctx, B[b]);
@@ -342,8 +331,23 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
         }
         if (ncoop > 0) {
             PM_TRY(coop_alloc(ctx, ncoop));
-            PM_CUDA(cudaMemcpy(ctx->coop_boxes, tab.data(), sizeof(CoopBox) * ncoop, cudaMemcpyHostToDevice));
+            // on the stream of the graph that reads it, and done before the table goes
+            PM_CUDA(cudaMemcpyAsync(ctx->coop_boxes, tab.data(), sizeof(CoopBox) * ncoop, cudaMemcpyHostToDevice,
+                                    ctx->batch_stream));
+            PM_CUDA(cudaStreamSynchronize(ctx->batch_stream));
         }
+    }
+    // flags of the boxes whose coarse levels are cluster launches (these and the cooperative boxes share
+    // one array: either form serves all boxes of a call).  Written before each graph launch, on the
+    // graph's stream; only the captured launches read them.
+    std::vector<int> cluster_idx(nbox, -1);
+    int ncluster = 0;
+    for (int b = 0; b < nbox; ++b)
+        if (B[b].active && B[b].cluster) cluster_idx[b] = ncluster++;
+    if (ncluster > 0) {
+        PM_TRY(coop_alloc(ctx, ncluster));
+        for (int b = 0; b < nbox; ++b)
+            if (cluster_idx[b] >= 0) B[b].cluster_active = ctx->coop_active + cluster_idx[b];
     }
     {
         std::vector<int> act;
@@ -566,7 +570,7 @@ pm_status mg_solve_batched(pm_ctx* ctx, int nbox, const int* nn, const double* c
                 R.st = PM_ERR_NOCONV;
                 break;
             }
-            x.cluster_active = nullptr;  // its flag may be down
+            x.cluster_active = nullptr;  // its flag is down
             R.active = true;
             box_iteration(&x, R);
             PM_CUDA(cudaStreamSynchronize(R.w->stream));
