@@ -265,9 +265,15 @@ extern "C" pm_status pm_create(pm_ctx** out, int device, void* stream, const pm_
         pm_destroy(ctx);
         return PM_ERR_OOM;
     }
-    cudaMemset(ctx->flag, 0, sizeof(int) * 4);
-    cudaMemset(ctx->red_partials, 0, sizeof(double) * kPartialsDoubles);  // partials and their counter
-    cudaMemset(ctx->red_out, 0, sizeof(double) * 64);
+    // cleared before the handle is out: the context's stream may be one that the legacy stream is not
+    // ordered before
+    if (cudaMemset(ctx->flag, 0, sizeof(int) * 4) != cudaSuccess ||
+        cudaMemset(ctx->red_partials, 0, sizeof(double) * kPartialsDoubles) != cudaSuccess ||  // with the tickets
+        cudaMemset(ctx->red_out, 0, sizeof(double) * 64) != cudaSuccess ||
+        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        pm_destroy(ctx);
+        return PM_ERR_CUDA;
+    }
     *out = ctx;
     return PM_OK;
 }

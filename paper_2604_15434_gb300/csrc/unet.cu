@@ -784,10 +784,15 @@ extern "C" pm_status pm_unet_create(pm_ctx* ctx, pm_unet** out)
             return st;
         }
     }
-    cudaMemset(u->p, 0, u->np * sizeof(float));
-    cudaMemset(u->g, 0, u->np * sizeof(float));
-    cudaMemset(u->m, 0, u->np * sizeof(float));
-    cudaMemset(u->v, 0, u->np * sizeof(float));
+    // cleared before the handle is out: the context's stream may be one that the legacy stream is not
+    // ordered before
+    for (float* p : {u->p, u->g, u->m, u->v})
+        if (cudaMemset(p, 0, u->np * sizeof(float)) != cudaSuccess) st = PM_ERR_CUDA;
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) st = PM_ERR_CUDA;
+    if (st != PM_OK) {
+        pm_unet_destroy(u);
+        return st;
+    }
     *out = u;
     return PM_OK;
 }
