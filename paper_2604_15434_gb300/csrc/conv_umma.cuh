@@ -130,13 +130,24 @@ constexpr int kUmBars = 2 * kUmMaxSlots + 2 * 32;
 
 // dynamic shared memory of k_conv3d_umma for Cin input channels, NT outputs and `slots` patch planes:
 // the resident weights, the planes, the barriers, the tensor-memory address, a failure flag, biases
-inline size_t umma_smem(int nt, int cin, int slots)
+constexpr size_t umma_smem(int nt, int cin, int slots)
 {
     return (size_t)9 * (cin / 16) * 2 * 3 * nt * 16 + (size_t)slots * (cin / 16) * kUmPP * 32 + kUmBars * 8 + 16 + nt * 4;
 }
 
 // shared memory for each of `blocks` blocks on an SM (1 KB per block is the system's)
 inline size_t umma_budget(int blocks) { return (size_t)(228 / blocks - 1) * 1024; }
+
+// Output channels per launch (16, 32, 48 or 64) of a layer of ci inputs and co outputs: the widest slice
+// whose resident weights fit beside two patch planes; 0 where the kernel does not take the layer.  fused:
+// a launch with an UmmaFuse, whose one instantiation has 16.
+constexpr int umma_slice(int ci, int co, bool fused)
+{
+    if (ci % 16 != 0 || co % 16 != 0) return 0;
+    int nt = fused ? 16 : co;
+    while ((nt > 64 || umma_smem(nt, ci, 2) > (size_t)227 * 1024) && nt % 32 == 0) nt /= 2;
+    return nt <= 64 && umma_smem(nt, ci, 2) <= (size_t)227 * 1024 ? nt : 0;
+}
 
 // Where a convolution's input comes from and what else its epilogue makes (forward passes that keep
 // no activations for a backward pass; null / 0 otherwise).

@@ -29,8 +29,13 @@ namespace pmeft {
 struct ConvSpec {
     int ci, co, level;
 };
-static const ConvSpec kConvs[10] = {{16, 16, 0}, {16, 16, 0}, {16, 32, 1}, {32, 32, 1}, {32, 64, 2},
-                                    {64, 64, 2}, {96, 32, 1}, {32, 32, 1}, {48, 16, 0}, {16, 16, 0}};
+static constexpr ConvSpec kConvs[10] = {{16, 16, 0}, {16, 16, 0}, {16, 32, 1}, {32, 32, 1}, {32, 64, 2},
+                                        {64, 64, 2}, {96, 32, 1}, {32, 32, 1}, {48, 16, 0}, {16, 16, 0}};
+// the layers that a forward pass may fuse (unet_fused): input, the two upsampled skips, head
+static_assert(umma_slice(kConvs[0].ci, kConvs[0].co, true) == 16 && umma_slice(kConvs[6].ci, kConvs[6].co, true) == 16 &&
+                  umma_slice(kConvs[8].ci, kConvs[8].co, true) == 16 &&
+                  umma_slice(kConvs[9].ci, kConvs[9].co, true) == kConvs[9].co,
+              "every fused layer has a tcgen05 launch");
 
 static long long conv_params(int i) { return 27LL * kConvs[i].ci * kConvs[i].co + kConvs[i].co; }
 static long long total_params()
@@ -450,20 +455,16 @@ static void launch_umma(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_
         mask_off, ctx->flag + 2, fuse);
 }
 
-// In slices of NT output channels whose resident weights fit beside two patch planes.  Returns false
-// (nothing launched) where it does not apply.
+// In slices of NT output channels (umma_slice).  Returns false (nothing launched) where it does not apply.
 static bool conv_umma(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off, int ci, const __nv_bfloat16* w,
                       int co, const float* bias, __nv_bfloat16* out, int out_ld, int out_off, int n, bool relu,
                       const __nv_bfloat16* mask, int mask_ld, int mask_off, const UmmaFuse& fuse)
 {
-    if (ctx->conv_path != 1 || n < kUmTY || n % kUmTY != 0 || ci % 16 != 0 || co % 16 != 0) return false;
-    int nt = co;  // the widest slice (at most 64 outputs) whose weights fit
-    while ((nt > 64 || umma_smem(nt, ci, 2) > (size_t)227 * 1024) && nt % 32 == 0) nt /= 2;
-    if (nt > 64 || umma_smem(nt, ci, 2) > (size_t)227 * 1024) return false;
+    const bool fused = fuse.half || fuse.up || fuse.T;
+    const int nt = umma_slice(ci, co, fused);
+    if (ctx->conv_path != 1 || n < kUmTY || n % kUmTY != 0 || nt == 0 || (fuse.T && co != nt)) return false;
     for (int co0 = 0; co0 < co; co0 += nt) {
         const bool two = umma_smem(nt, ci, 4) <= umma_budget(2);
-        const bool fused = fuse.half || fuse.up || fuse.T;
-        if (fused && nt != 16) return false;
         const auto launch = fused      ? (two ? launch_umma<16, 2, true> : launch_umma<16, 1, true>)
                             : nt == 16   ? (two ? launch_umma<16, 2> : launch_umma<16, 1>)
                             : nt == 32 ? (two ? launch_umma<32, 2> : launch_umma<32, 1>)
@@ -475,8 +476,9 @@ static bool conv_umma(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_of
     return true;
 }
 
-// forward conv launcher (also the backward-data conv with a mask)
-static void conv_fwd(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off, int ci, const __nv_bfloat16* w,
+// forward conv launcher (also the backward-data conv with a mask).  A fused input or head is known to the
+// tcgen05 kernel only: where that does not apply, nothing is launched and the call fails.
+static pm_status conv_fwd(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off, int ci, const __nv_bfloat16* w,
                      int co, const float* bias, __nv_bfloat16* out, int out_ld, int out_off, int n, bool relu,
                      const __nv_bfloat16* mask = nullptr, int mask_ld = 0, int mask_off = 0,
                      const UmmaFuse& fuse = {})
@@ -486,7 +488,12 @@ static void conv_fwd(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off
     if (conv_umma(ctx, in, in_ld, in_off, ci, w, co, bias, out, out_ld, out_off, n, relu, mask, mask_ld, mask_off,
                   fuse)) {
         ctx->end();
-        return;
+        return PM_OK;
+    }
+    if (fuse.half || fuse.up || fuse.T) {
+        ctx->end();
+        ctx->set_error("fused convolution: no kernel for this layer");
+        return PM_ERR_CUDA;
     }
     // grids of 16^3 and up whose weights fit next to the patch in shared memory take the
     // persistent tiled kernel, the rest the per-128-voxel kernel
@@ -536,6 +543,7 @@ static void conv_fwd(pm_ctx* ctx, const __nv_bfloat16* in, int in_ld, int in_off
 #undef PM_CONV_CASE
     }
     ctx->end();
+    return PM_OK;
 }
 
 template <int CO, int KX>
@@ -634,7 +642,7 @@ static pm_status unet_forward(pm_unet* u, const double* delta, int n, double aB0
     k_pack_input<<<blocks_for(ctx, v0), 256, 0, ctx->stream>>>(delta, (int)v0, (float)aB0, (float)aM0, (float)a, in_ld,
                                                                A.in);
     ctx->end();
-    conv_fwd(ctx, A.in, in_ld, 0, 16, u->wf[0], 16, bias_of(u, 0), A.y0, 16, 0, n, true, nullptr, 0, 0, half);
+    PM_TRY(conv_fwd(ctx, A.in, in_ld, 0, 16, u->wf[0], 16, bias_of(u, 0), A.y0, 16, 0, n, true, nullptr, 0, 0, half));
     conv_fwd(ctx, A.y0, 16, 0, 16, u->wf[1], 16, bias_of(u, 1), s1, s1_ld, s1_off, n, true);
     ctx->begin(PM_K_PM);
     k_pool2<<<blocks_for(ctx, v0 / 8 * 16), 256, 0, ctx->stream>>>(s1, s1_ld, s1_off, 16, n, A.p1);
@@ -651,15 +659,15 @@ static pm_status unet_forward(pm_unet* u, const double* delta, int n, double aB0
         k_up2<<<blocks_for(ctx, v0 / 8 * 64), 256, 0, ctx->stream>>>(A.y5, 64, n2, A.cat2, 96, 0);
         ctx->end();
     }
-    conv_fwd(ctx, s2, s2_ld, 0, 96, u->wf[6], 32, bias_of(u, 6), A.y6, 32, 0, n1, true, nullptr, 0, 0, up1);
+    PM_TRY(conv_fwd(ctx, s2, s2_ld, 0, 96, u->wf[6], 32, bias_of(u, 6), A.y6, 32, 0, n1, true, nullptr, 0, 0, up1));
     conv_fwd(ctx, A.y6, 32, 0, 32, u->wf[7], 32, bias_of(u, 7), A.y7, 32, 0, n1, true);
     if (!f0) {
         ctx->begin(PM_K_PM);
         k_up2<<<blocks_for(ctx, v0 * 32), 256, 0, ctx->stream>>>(A.y7, 32, n1, A.cat1, 48, 0);
         ctx->end();
     }
-    conv_fwd(ctx, s1, s1_ld, 0, 48, u->wf[8], 16, bias_of(u, 8), A.y8, 16, 0, n, true, nullptr, 0, 0, up0);
-    conv_fwd(ctx, A.y8, 16, 0, 16, u->wf[9], 16, bias_of(u, 9), A.y9, 16, 0, n, true, nullptr, 0, 0, head);
+    PM_TRY(conv_fwd(ctx, s1, s1_ld, 0, 48, u->wf[8], 16, bias_of(u, 8), A.y8, 16, 0, n, true, nullptr, 0, 0, up0));
+    PM_TRY(conv_fwd(ctx, A.y8, 16, 0, 16, u->wf[9], 16, bias_of(u, 9), A.y9, 16, 0, n, true, nullptr, 0, 0, head));
     if (!f0) {
         ctx->begin(PM_K_PM);
         k_head<<<blocks_for(ctx, v0), 256, 0, ctx->stream>>>(A.y9, u->p + u->off[10], (int)v0, A.that);
