@@ -16,6 +16,7 @@
 
 #include "internal.cuh"
 #include "cell64.cuh"
+#include "sums.cuh"
 #include "sweep_fused.cuh"
 #include "sweep_pair.cuh"
 #include "sweep_col.cuh"
@@ -935,67 +936,6 @@ __global__ void __launch_bounds__(kExactThreads) k_coarsest_exact(T* __restrict_
 }
 
 // ------------------------------------------------------------------ misc
-
-// sum of x, four loads in flight per thread: FP32 data (the library's own buffers) by 16-byte
-// loads in FP32 per-thread sums (a few hundred terms each), FP64 across threads; FP64 data (the
-// caller's density among it) by aligned 8-byte loads, one FP64 addition per element
-template <typename T>
-__global__ void __launch_bounds__(256) k_sum(const T* __restrict__ x, size_t total, double* __restrict__ partials,
-                                             double* __restrict__ fin_out)
-{
-    constexpr int W = sizeof(T) == 4 ? 4 : 1;
-    struct alignas(W * sizeof(T)) Vec {
-        T e[W];
-    };
-    const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-    const size_t nv = total / W;  // total is a multiple of 512
-    const Vec* xv = reinterpret_cast<const Vec*>(x);
-    T a[4] = {T(0), T(0), T(0), T(0)};
-    size_t c = tid;
-    for (; c + 3 * stride < nv; c += 4 * stride) {
-        Vec q[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) q[k] = xv[c + k * stride];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int e = 0; e < W; ++e) a[k] += q[k].e[e];
-    }
-    for (; c < nv; c += stride) {
-        const Vec q = xv[c];
-#pragma unroll
-        for (int e = 0; e < W; ++e) a[0] += q.e[e];
-    }
-    const T v[1] = {(a[0] + a[1]) + (a[2] + a[3])};
-    block_sums<1>(v, partials, fin_out, (double)total);
-}
-
-// sum of (x - mean)^2 with the mean read from the device (sums[1], as k_sum leaves it)
-__global__ void __launch_bounds__(256) k_sum_centred(const double* __restrict__ x, size_t total,
-                                                     const double* __restrict__ sums, double* __restrict__ partials,
-                                                     double* __restrict__ fin_out)
-{
-    const double mean = sums[1];
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; c + 3 * stride < total; c += 4 * stride) {
-        double q[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) q[k] = x[c + k * stride];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const double d = q[k] - mean;
-            a[k] += d * d;
-        }
-    }
-    for (; c < total; c += stride) {
-        const double d = x[c] - mean;
-        a[0] += d * d;
-    }
-    const double v[1] = {(a[0] + a[1]) + (a[2] + a[3])};
-    block_sums<1>(v, partials, fin_out, 1.0);
-}
 
 template <typename T>
 __global__ void k_sub_mean(T* __restrict__ x, size_t total, const double* __restrict__ sums)
