@@ -11,7 +11,7 @@
 // neighbour block's ghost plane (distributed shared memory), so one cluster barrier per half-sweep
 // separates everything.  The sums of a level's gauge shift go to every block's shared memory at the
 // barrier that ends the restriction.  Arithmetic per cell is that of half_sweep_cell, residual_cell,
-// fas_rhs_cell and prolong_children; the sums are float-float across a warp, FP64 across warps.
+// fas_rhs_cell and prolong_children; the sums are FP64, as those of the level-by-level kernels.
 //
 // One launch takes 55 us (the launches it replaces took some 160 us of a V-cycle): 12 on each side
 // of it for the 32^3 sweeps, 14 for the coarsest solve.  What bounds it is latency: a few hundred
@@ -139,20 +139,6 @@ __device__ __forceinline__ Stencil<float> cl_stencil(const float* lo, const floa
     s.exz = hi[r + ip] - lo[r + ip] - hi[r + im] + lo[r + im];
     s.eyz = hi[rp + i] - lo[rp + i] - hi[rm + i] + lo[rm + i];
     return s;
-}
-
-// sum over the warp in float-float (48 bits), as a double
-__device__ __forceinline__ double cl_warp_sum(float v)
-{
-    float hi = v, lo = 0.f;
-    for (int d = 16; d > 0; d >>= 1) {
-        const float h = __shfl_xor_sync(0xffffffffu, hi, d), l = __shfl_xor_sync(0xffffffffu, lo, d);
-        const float s = __fadd_rn(hi, h), b = __fsub_rn(s, hi);
-        const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(h, b));
-        lo = __fadd_rn(__fadd_rn(lo, l), e);
-        hi = s;
-    }
-    return (double)hi + (double)lo;
 }
 
 // The four children in one fine plane of coarse column (I, J): near and far are the coarse planes
@@ -287,18 +273,19 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
             __syncthreads();
         }
     };
-    // a block's residual sum and unfloored count into wsum/wcnt[0]: per-thread values in, valid
-    // after the caller's next barrier
-    auto block_sum = [&](float v, int unfl) {
-        const double s = cl_warp_sum(v);
-        const int n = __reduce_add_sync(0xffffffffu, unfl);
-        if (lane == 0) {
-            cl_s[0].wsum[wid] = s;
-            cl_s[0].wcnt[wid] = n;
+    // a block's residual sum and unfloored count into wsum/wcnt[0]: the values of its first nw warps in,
+    // valid after the caller's next barrier
+    auto block_sum = [&](double v, int unfl, int nw) {
+        if (wid < nw) {
+            const double s = warp_sum(v);
+            const int n = __reduce_add_sync(0xffffffffu, unfl);
+            if (lane == 0) {
+                cl_s[0].wsum[wid] = s;
+                cl_s[0].wcnt[wid] = n;
+            }
         }
         __syncthreads();
         if (wid == 0) {
-            constexpr int nw = kClThreads / 32;
             const double a = warp_sum(lane < nw ? cl_s[0].wsum[lane] : 0.0);
             const int c = __reduce_add_sync(0xffffffffu, lane < nw ? cl_s[0].wcnt[lane] : 0);
             if (lane == 0) {
@@ -334,7 +321,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
         for (int s = 0; s < (leg32 ? P.npost : P.npre); ++s) sweep32();
         if (leg32) break;
         {
-            float v = 0.f;
+            double v = 0.0;
             int un = 0;
 #pragma unroll 1
             for (int q = 0; q < 2; ++q)
@@ -348,10 +335,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                     const float r = cl_resid(cl_eval(s, k, 1024.f, P.nu, k.f), P.nu, fl);
                     cl_s[0].r32[p][c] = r;
                     cl_s[0].fl32[p][c] = fl;
-                    v += r;
+                    v += f2d_bits(r);
                     un += !fl;
                 }
-            block_sum(v, un);
+            block_sum(v, un, kClThreads / 32);
             share_sums(0);
             if (t < 256) {  // plane r of the 16^3 level; the gauge term waits for the sums
                 const int I = t & 15, J = t >> 4;
@@ -398,7 +385,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
             {
                 // the residual; each thread's pair and the row below it (eight lanes on) are the plane's four
                 // children of an 8^3 cell, whose part goes to block 0
-                float v = 0.f, su = 0.f, sb = 0.f;
+                double v = 0.0;
+                float sr = 0.f, su = 0.f, sb = 0.f;
                 int un = 0, cnt = 0;
                 if (t < 128) {
 #pragma unroll 1
@@ -407,13 +395,15 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                         const ClCell k = cl_s[0].c16[c];
                         const Stencil<float> s = cl_stencil<16>(cl_s[0].u16[b16][0], cl_s[0].u16[b16][1], cl_s[0].u16[b16][2], i, j16);
                         bool fl;
-                        v += cl_resid(cl_eval(s, k, 256.f, P.nu, k.f), P.nu, fl);
+                        const float r = cl_resid(cl_eval(s, k, 256.f, P.nu, k.f), P.nu, fl);
+                        v += f2d_bits(r);
+                        sr += r;
                         su += s.c0;
                         sb += cl_s[0].bg16[1][c];
                         un += !fl;
                         cnt += fl ? 8 : min((int)cl_s[0].km16[c], 8);
                     }
-                    const float v2 = v + __shfl_down_sync(0xffffffffu, v, 8);
+                    sr += __shfl_down_sync(0xffffffffu, sr, 8);
                     su += __shfl_down_sync(0xffffffffu, su, 8);
                     sb += __shfl_down_sync(0xffffffffu, sb, 8);
                     cnt += __shfl_down_sync(0xffffffffu, cnt, 8);
@@ -422,13 +412,13 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                         ClSmem* o = cl.map_shared_rank(&cl_s[0], 0);
                         const int h = rank & 1, c = (rank >> 1) * 64 + (j16 >> 1) * 8 + m16;
                         o->h8[0][h][c] = su;
-                        o->h8[1][h][c] = v2;
+                        o->h8[1][h][c] = sr;
                         o->h8[2][h][c] = sb;
                         o->hc8[h][c] = (uint8_t)cnt;
                         o->hn8[h][c] = (uint8_t)n2;
                     }
                 }
-                block_sum(v, un);
+                block_sum(v, un, 4);
                 share_sums(1);
                 cl.sync();
             }
@@ -455,7 +445,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
 #pragma unroll 1
                     for (int s = 0; s < (leg8 ? P.npost : P.npre); ++s) sweep8();
                     if (leg8) break;
-                    float v = 0.f;
+                    double v = 0.0;
                     int un = 0;
                     if (t < 512) {
                         const int i = t & 7, j = (t >> 3) & 7, k = t >> 6;
@@ -464,10 +454,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                         const float r = cl_resid(cl_eval(stencil8(cl_s[0].u8[b8], i, j, k), c, 64.f, P.nu, c.f), P.nu, fl);
                         cl_s[0].r8[t] = r;
                         cl_s[0].fl8[t] = fl;
-                        v = r;
+                        v = f2d_bits(r);
                         un = !fl;
                     }
-                    block_sum(v, un);
+                    block_sum(v, un, kClThreads / 32);
                     if (t < 64) {  // the 4^3 level
                         const float gm = cl_s[0].wcnt[0] > 0 ? (float)(cl_s[0].wsum[0] / (double)cl_s[0].wcnt[0]) : 0.f;
                         const int I = t & 3, J = (t >> 2) & 3, K = t >> 4;
