@@ -74,13 +74,13 @@ __device__ __forceinline__ Eval64 eval64(const Stencil<double>& s, double nu1, d
     return o;
 }
 
-// a < b for b >= +0 on the integer pipe, false for a NaN of either sign: among the negative values' bits,
-// those above -infinity's are NaNs (and the NaN that an operation makes here has its sign set).  -0, which
-// a discriminant is only where it underflows, counts as negative.
+// a < b for b >= +0 on the integer pipe, false for a NaN of either sign: among the negative values' high
+// words, those above -infinity's are NaNs (the NaN that an operation makes here has its sign set; a is the
+// result of one, so a NaN is quiet and its high word says so).  -0, which a discriminant is only where it
+// underflows, counts as negative.
 __device__ __forceinline__ bool below64(double a, double b)
 {
-    const long long x = __double_as_longlong(a);
-    return x < __double_as_longlong(b) && (unsigned long long)x <= 0xfff0000000000000ull;
+    return __double_as_longlong(a) < __double_as_longlong(b) && (unsigned)__double2hiint(a) <= 0xfff00000u;
 }
 __device__ __forceinline__ bool screened64(const KW64& w) { return (__double_as_longlong(w.m2) << 1) != 0; }
 
@@ -94,9 +94,9 @@ __device__ __forceinline__ double update64(const Eval64& o, const K64& k, const 
     if (screened64(w)) {
         if (below64(o.D, k.Df)) return -gap64(o, k.ih2, w.lsat) * k.h2o6;
         const double sq = sqrt(o.D), ssq = k.sp < 0.0 ? -sq : sq;
-        // Ep and ssq of one sign (compared by their sign bits): -2G/(Ep + ssq), else, and for Ep = 0 of
-        // either sign, the other form
-        if ((__double2hiint(o.Ep) ^ __double2hiint(k.sp)) >= 0 && (__double_as_longlong(o.Ep) << 1) != 0) {
+        // Ep and ssq of one sign (by their sign bits): -2G/(Ep + ssq), else, and for Ep = 0 of either sign,
+        // the other form
+        if ((__double2hiint(o.Ep) ^ (__double2hiint(k.sp) & (int)0x80000000)) > 0) {
             num = -2.0 * o.G;
             den = o.Ep + ssq;
         } else {
