@@ -212,7 +212,7 @@ struct Workspace {
                                    // iterate out of place)
     uint32_t* coef_test = nullptr; // coefficients of a caller's background (pm_mg_sweep_f32, mode > 100)
     double* psi = nullptr;         // scratch n^3 (Poisson output / total potential)
-    double* grad = nullptr;        // scratch 5 n^3: the grid force [n^3][4] and the total potential (force kernels)
+    double* grad = nullptr;        // scratch 4 n^3: the grid force [n^3][4] (force kernels)
     double* delta = nullptr;       // scratch n^3 (pm_step)
     long long* acc = nullptr;      // int64 fixed-point deposit grid
     cufftHandle plan_r2c = 0, plan_c2r = 0;

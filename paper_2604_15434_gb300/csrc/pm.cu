@@ -212,9 +212,9 @@ __global__ void k_f2d(const float* __restrict__ x, size_t total, double* __restr
         y[c] = (double)x[c];
 }
 
-// Psi = psiN + xi chi on the grid, rounded as written.
-__global__ void __launch_bounds__(256) k_psi_total(const double* __restrict__ psiN, const double* __restrict__ chi,
-                                                   double xi, size_t total, double* __restrict__ psi)
+// Psi = psiN + xi chi on the grid, rounded as written; psi may be psiN.
+__global__ void __launch_bounds__(256) k_psi_total(const double* psiN, const double* __restrict__ chi, double xi,
+                                                   size_t total, double* psi)
 {
     for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < total; c += (size_t)gridDim.x * blockDim.x)
         psi[c] = __dadd_rn(psiN[c], __dmul_rn(xi, chi[c]));
@@ -453,22 +453,22 @@ pm_status poisson32(pm_ctx* ctx, const double* delta, int n, double fac, double*
 }
 
 // g = -grad(psiN + xi chi) at each particle (Eq. force, Sec. 3.5.2; psiN alone when chi is null): the
-// total potential and its gradient on the grid (workspace: [n^3][4] force, then [n^3] Psi), then the
-// CIC interpolation of the grid force.
+// total potential (in the workspace's psi, in place where psiN is that) and its gradient on the grid
+// (workspace: [n^3][4]), then the CIC interpolation of the grid force.
 pm_status interp_force(pm_ctx* ctx, const double* psiN, const double* chi, double xi, int n, const double* pos,
                        long long np, double* acc)
 {
     Workspace* w = nullptr;
     PM_TRY(get_workspace(ctx, n, &w));
     const size_t cells = (size_t)n * n * n;
-    if (!w->grad) PM_CUDA(cudaMalloc(&w->grad, 5 * cells * sizeof(double)));
+    if (!w->grad) PM_CUDA(cudaMalloc(&w->grad, 4 * cells * sizeof(double)));
     const double* psi = psiN;
     if (chi) {
-        double* sum = w->grad + 4 * cells;
+        if (!w->psi) PM_CUDA(cudaMalloc(&w->psi, cells * sizeof(double)));
         ctx->begin(PM_K_PM, false, 0);
-        k_psi_total<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psiN, chi, xi, cells, sum);
+        k_psi_total<<<grid_for(ctx, cells), kThreads, 0, ctx->stream>>>(psiN, chi, xi, cells, w->psi);
         ctx->end();
-        psi = sum;
+        psi = w->psi;
     }
     const bool four = ctx->prm.grad_order != 2;
     const int lg = __builtin_ctz(n);
