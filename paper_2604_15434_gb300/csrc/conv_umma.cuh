@@ -18,8 +18,9 @@
 // Roles: three warps copy input planes, one thread watches the barriers, one issues MMAs, two groups of
 // four warps read finished output planes back in turn; they meet only at mbarriers, so copies, tensor
 // core and epilogue run at their own pace.  What bounds it is shared memory: an MMA of N = 48 reads 4 KB
-// of A and 1.5 KB of B and takes 57 cycles, one of N = 96 78.  When the same warps did everything in
-// turn, plane by plane, the tensor pipe was 21 to 35% busy (now 27 to 43).  Moving the window of output
+// of A and 1.5 KB of B and takes 57 cycles, one of N = 96 78.  The tensor pipe is busy 23% of the time for
+// 16 -> 16 channels at 256^3, 35 for 48 -> 16, 43 for 32 -> 32 at 128^3; for 16 -> 16 at 128^3 17 to 20 (18 when
+// the same warps did everything in turn, plane by plane, in 85 us a layer; now 64).  Moving the window of output
 // planes costs the tensor core some 500 cycles more per input plane, which a second block on the SM
 // fills where two fit (16 -> 16 channels at 256^3: one block 0.52 ms, two 0.36).
 // Before -> now: 256^3 16 -> 16 channels 0.41 -> 0.36 ms, 48 -> 16 1.36 -> 0.80; 128^3 96 -> 32 0.79 -> 0.54,
@@ -39,7 +40,10 @@ constexpr int kUmPP = kUmPX * kUmPY;                       // 180 voxels per pat
 constexpr int kUmEpi = 128, kUmLoad = 96;                  // threads of an epilogue group, copying threads
 constexpr int kUmThreads = 2 * kUmEpi + 64 + kUmLoad;      // warps 0-3 and 4-7 (epilogue), 8 (MMA issue), 9-11
                                                            // (copies), 12 (lookout)
-constexpr long long kUmSpin = 1ll << 22;                   // bound on an mbarrier wait (polls)
+// Bound on a wait, in polls.  A poll is a shared-memory round trip at least (some 30 cycles; try_wait may sleep
+// longer), so 2^22 of them are 60 ms or more.  The longest wait of a working launch is for the MMAs of the
+// planes in flight: at most eight planes of 54 MMAs of 78 cycles, 34 k cycles or 16 us.
+constexpr long long kUmSpin = 1ll << 22;
 
 __device__ __forceinline__ uint32_t um_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

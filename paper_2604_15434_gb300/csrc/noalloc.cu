@@ -30,7 +30,7 @@ struct StaticSlot {
 static std::mutex g_static_mu;
 static StaticSlot g_static_slots[64];
 
-void launch_deposit_on(cudaStream_t s, int sms, const double* pos, long long np, int n, unsigned long long* acc);
+void launch_deposit_on(cudaStream_t s, const double* pos, long long np, int n, unsigned long long* acc);
 void launch_density_on(cudaStream_t s, int sms, const long long* acc, int n, long long np, double* delta, int* flag);
 
 }  // namespace pmeft
@@ -66,7 +66,7 @@ extern "C" pm_status pm_deposit_cic_static(const double* pos, long long np, int 
     if (cudaMemsetAsync(slot.acc, 0, cells * sizeof(unsigned long long), s) != cudaSuccess) return PM_ERR_CUDA;
     if (cudaMemsetAsync(slot.flag, 0, sizeof(int), s) != cudaSuccess) return PM_ERR_CUDA;
     // each launch is checked at once, so that a failure is reported by the call that made it
-    launch_deposit_on(s, slot.sms, pos, np, n, slot.acc);
+    launch_deposit_on(s, pos, np, n, slot.acc);
     if (cudaGetLastError() != cudaSuccess) return PM_ERR_CUDA;
     launch_density_on(s, slot.sms, (const long long*)slot.acc, n, np, delta, slot.flag);
     if (cudaGetLastError() != cudaSuccess) return PM_ERR_CUDA;

@@ -20,9 +20,10 @@
 // (Columns marched in z with chunks cut to the number of blocks took 1.03 ms for the ten layers
 // where this takes 1.6, but moved the gradient by up to 2e-5.)
 //
-// What bounds it now is the rate of mma.sync, about one m16n8k16 per four cycles and SM.  The
-// tcgen05 shapes gain little at these channel counts: their M of 64 or 128 rows is 3 or 6 z taps of
-// 16 channels, read again from shared memory for every in-plane tap.
+// No pipe is full now (16 and 48 -> 16 channels at 128^3: tensor 34 and 40%, issue 47 and 54%, L1 51 and
+// 60%; one m16n8k16 per six cycles and SM): it is the latency of ldmatrix and mma.sync at 7 to 12 warps
+// per SM.  The tcgen05 shapes gain little at these channel counts: their M of 64 or 128 rows is 3 or
+// 6 z taps of 16 channels, read again from shared memory for every in-plane tap.
 // Measured at 128^3: 48 -> 16 channels 2.82 -> 0.42 ms, 96 -> 32 at 64^3 1.33 -> 0.23 ms, all ten
 // layers with their biases and reductions 9.3 -> 1.7 ms of a 12.0 ms training step.
 #pragma once
