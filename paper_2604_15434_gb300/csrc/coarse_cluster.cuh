@@ -56,7 +56,7 @@ struct ClSmem {
     ClCell c8[512];
     float u4[64], ur4[64], bg4[64], f4[64];
     CoarsestSmem<float> cs;
-    double wsum[kClThreads / 32], csum[2][kClBlocks];  // csum, ccnt: of the 32^3 and of the 16^3 level
+    double wsum[128], csum[2][kClBlocks];  // csum, ccnt: of the 32^3 and of the 16^3 level
     int wcnt[kClThreads / 32], ccnt[2][kClBlocks];
     float gm;
     uint8_t km32[2][1024], fl32[2][1024], km16[256], nun16[256], km8[512], fl8[512], km4[64];
@@ -273,21 +273,24 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
             __syncthreads();
         }
     };
-    // a block's residual sum and unfloored count into wsum/wcnt[0]: the values of its first nw warps in,
-    // valid after the caller's next barrier
-    auto block_sum = [&](double v, int unfl, int nw) {
-        if (wid < nw) {
-            const double s = warp_sum(v);
-            const int n = __reduce_add_sync(0xffffffffu, unfl);
-            if (lane == 0) {
-                cl_s[0].wsum[wid] = s;
-                cl_s[0].wcnt[wid] = n;
-            }
+    // a block's residual sum and unfloored count into wsum/wcnt[0]: `count` values in shared memory (a
+    // multiple of 128) and each thread's unfloored cells in.  FP64 additions, 16 cycles each per warp and SM,
+    // are what it costs: four warps and then one add up columns, so that there is one shuffle tree and not one per warp.
+    auto block_sum = [&](const float* v, int count, int unfl) {
+        const int n = __reduce_add_sync(0xffffffffu, unfl);
+        if (lane == 0) cl_s[0].wcnt[wid] = n;
+        __syncthreads();
+        if (t < 128) {
+            double s = f2d_bits(v[t]);
+#pragma unroll 4
+            for (int i = t + 128; i < count; i += 128) s += f2d_bits(v[i]);
+            cl_s[0].wsum[t] = s;
         }
         __syncthreads();
         if (wid == 0) {
-            const double a = warp_sum(lane < nw ? cl_s[0].wsum[lane] : 0.0);
-            const int c = __reduce_add_sync(0xffffffffu, lane < nw ? cl_s[0].wcnt[lane] : 0);
+            const double a = warp_sum((cl_s[0].wsum[lane] + cl_s[0].wsum[lane + 32]) +
+                                      (cl_s[0].wsum[lane + 64] + cl_s[0].wsum[lane + 96]));
+            const int c = __reduce_add_sync(0xffffffffu, lane < kClThreads / 32 ? cl_s[0].wcnt[lane] : 0);
             if (lane == 0) {
                 cl_s[0].wsum[0] = a;
                 cl_s[0].wcnt[0] = c;
@@ -321,7 +324,6 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
         for (int s = 0; s < (leg32 ? P.npost : P.npre); ++s) sweep32();
         if (leg32) break;
         {
-            double v = 0.0;
             int un = 0;
 #pragma unroll 1
             for (int q = 0; q < 2; ++q)
@@ -335,10 +337,9 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                     const float r = cl_resid(cl_eval(s, k, 1024.f, P.nu, k.f), P.nu, fl);
                     cl_s[0].r32[p][c] = r;
                     cl_s[0].fl32[p][c] = fl;
-                    v += f2d_bits(r);
                     un += !fl;
                 }
-            block_sum(v, un, kClThreads / 32);
+            block_sum(cl_s[0].r32[0], 2048, un);
             share_sums(0);
             if (t < 256) {  // plane r of the 16^3 level; the gauge term waits for the sums
                 const int I = t & 15, J = t >> 4;
@@ -385,7 +386,6 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
             {
                 // the residual; each thread's pair and the row below it (eight lanes on) are the plane's four
                 // children of an 8^3 cell, whose part goes to block 0
-                double v = 0.0;
                 float sr = 0.f, su = 0.f, sb = 0.f;
                 int un = 0, cnt = 0;
                 if (t < 128) {
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                         const Stencil<float> s = cl_stencil<16>(cl_s[0].u16[b16][0], cl_s[0].u16[b16][1], cl_s[0].u16[b16][2], i, j16);
                         bool fl;
                         const float r = cl_resid(cl_eval(s, k, 256.f, P.nu, k.f), P.nu, fl);
-                        v += f2d_bits(r);
+                        cl_s[0].rs16[c] = r;
                         sr += r;
                         su += s.c0;
                         sb += cl_s[0].bg16[1][c];
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                         o->hn8[h][c] = (uint8_t)n2;
                     }
                 }
-                block_sum(v, un, 4);
+                block_sum(cl_s[0].rs16, 256, un);
                 share_sums(1);
                 cl.sync();
             }
@@ -445,7 +445,6 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
 #pragma unroll 1
                     for (int s = 0; s < (leg8 ? P.npost : P.npre); ++s) sweep8();
                     if (leg8) break;
-                    double v = 0.0;
                     int un = 0;
                     if (t < 512) {
                         const int i = t & 7, j = (t >> 3) & 7, k = t >> 6;
@@ -454,10 +453,9 @@ __global__ void __launch_bounds__(kClThreads, 1) k_coarse_cluster(ClusterParams 
                         const float r = cl_resid(cl_eval(stencil8(cl_s[0].u8[b8], i, j, k), c, 64.f, P.nu, c.f), P.nu, fl);
                         cl_s[0].r8[t] = r;
                         cl_s[0].fl8[t] = fl;
-                        v = f2d_bits(r);
                         un = !fl;
                     }
-                    block_sum(v, un, kClThreads / 32);
+                    block_sum(cl_s[0].r8, 512, un);
                     if (t < 64) {  // the 4^3 level
                         const float gm = cl_s[0].wcnt[0] > 0 ? (float)(cl_s[0].wsum[0] / (double)cl_s[0].wcnt[0]) : 0.f;
                         const int I = t & 3, J = (t >> 2) & 3, K = t >> 4;
