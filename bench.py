@@ -426,7 +426,7 @@ def next_rows_leg(api, dev, stream):
     ms, dlt = timed(lambda: api.pm_deposit_cic(pos0, n, ctx=cp), 5)
     byt = 24 * n ** 3 + 24 * n ** 3
     out["deposit"] = {"ms": ms, "particles_per_s": n ** 3 / (ms * 1e-3), "gbs": byt / (ms * 1e-3) / 1e9,
-                      "frac_of_hbm": byt / (ms * 1e-3) / 1e9 / hbm, "bound": "L2 atomics"}
+                      "frac_of_hbm": byt / (ms * 1e-3) / 1e9 / hbm, "bound": "64-bit reductions (L1, L2)"}
     ms, psn = timed(lambda: api.poisson_solve(dlt, 1.0, 0.2, ctx=cp), 5)
     out["poisson_fft"] = {"ms": ms}
     acc = torch.empty_like(pos0)

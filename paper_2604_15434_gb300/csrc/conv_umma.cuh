@@ -18,7 +18,7 @@
 // Roles: three warps copy input planes, one thread watches the barriers, one issues MMAs, two groups of
 // four warps read finished output planes back in turn; they meet only at mbarriers, so copies, tensor
 // core and epilogue run at their own pace.  What bounds it is shared memory: an MMA of N = 48 reads 4 KB
-// of A and 1.5 KB of B and takes 57 cycles, one of N = 96 78.  The tensor pipe is busy 23% of the time for
+// of A and 1.5 KB of B and takes 57 cycles, one of N = 96 78.  The tensor pipe is busy 28% of the time for
 // 16 -> 16 channels at 256^3, 35 for 48 -> 16, 43 for 32 -> 32 at 128^3; for 16 -> 16 at 128^3 17 to 20 (18 when
 // the same warps did everything in turn, plane by plane, in 85 us a layer; now 64).  Moving the window of output
 // planes costs the tensor core some 500 cycles more per input plane, which a second block on the SM

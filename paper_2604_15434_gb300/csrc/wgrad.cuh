@@ -21,7 +21,7 @@
 // where this takes 1.6, but moved the gradient by up to 2e-5.)
 //
 // No pipe is full now (16 and 48 -> 16 channels at 128^3: tensor 34 and 40%, issue 47 and 54%, L1 51 and
-// 60%; one m16n8k16 per six cycles and SM): it is the latency of ldmatrix and mma.sync at 7 to 12 warps
+// 60%; one m16n8k16 per six cycles and SM): it is the latency of ldmatrix and mma.sync at 15 to 23 warps
 // per SM.  The tcgen05 shapes gain little at these channel counts: their M of 64 or 128 rows is 3 or
 // 6 z taps of 16 channels, read again from shared memory for every in-plane tap.
 // Measured at 128^3: 48 -> 16 channels 2.82 -> 0.42 ms, 96 -> 32 at 64^3 1.33 -> 0.23 ms, all ten
